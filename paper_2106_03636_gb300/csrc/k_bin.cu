@@ -396,7 +396,104 @@ __global__ void __launch_bounds__(kT) k_cell_sort(const RowGrid* __restrict__ gr
   }
 }
 
+// K3c: the drift-ordered view of every row (ZRow), one CTA per row, from the
+// sorted hits.  Bins of at least 1 cm, at most one per hit.  The sorted order
+// runs through the cell rows in drift order, so a chunk of cell rows is a
+// contiguous run of hits whose bins are a contiguous run too (its first bin
+// may be shared with the chunk before, whose hits come first): every chunk is
+// counted, scanned and scattered by itself in shared memory, its output range
+// is its input range, and the writes stay inside it.  Bound by memory: 8
+// bytes read (twice, the second time from L2), 12 + 4 per bin written per hit.
+constexpr int kZBins = 4096, kZThreads = 256;
+constexpr int kZBinWidth = 124;  // units: 1 cm at 2.58 cm/us
+__global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict__ grid, const int* __restrict__ rowMax,
+                                                      const int* __restrict__ cellStart, const int2* __restrict__ syz,
+                                                      ZRow* __restrict__ zrow, int4* __restrict__ bucket) {
+  __shared__ int s_cnt[kZBins + 1];
+  __shared__ int s_warp[kZThreads / 32];
+  const RowGrid g = grid[blockIdx.x];
+  ZRow z{};
+  z.start = g.start;
+  z.count = g.count;
+  if (g.count == 0) {
+    if (threadIdx.x == 0) zrow[blockIdx.x] = z;
+    return;
+  }
+  const float range = (float)((unsigned)rowMax[blockIdx.x] - (unsigned)g.zmin) + 1.f;
+  z.zmin = g.zmin;
+  z.nzb = max(1, min(min((int)(range * (1.f / kZBinWidth)), g.count), g.nz * (kZBins - 96)));
+  z.zinv = (float)z.nzb / range;
+  // expected hits of a whole row in a window (plus the bins' own width)
+  // against ~10 in the cells that cover it
+  const float perUnit = (float)g.count / range, binw = range / (float)z.nzb;
+  if (perUnit * (2 * kWinZ + binw) > 20.f) z.flags |= kZNFCells;
+  if (perUnit * (140.f + binw) > 12.f) z.flags |= kZFollowCells;
+  if (threadIdx.x == 0) zrow[blockIdx.x] = z;
+  char* mem = reinterpret_cast<char*>(bucket) + 16ll * g.start;
+  int2* yz = reinterpret_cast<int2*>(mem);
+  int* idx = reinterpret_cast<int*>(mem + 8ll * g.count);
+  int* bins = reinterpret_cast<int*>(mem + 12ll * g.count);
+  const float perCellRow = (float)g.cz * z.zinv * 1.0001f + 1.f;
+  const int izPer = max(1, (int)((float)(kZBins - 8) / perCellRow));
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int bL = -1;  // last bin of the chunks before
+  for (int iz0 = 0; iz0 < g.nz; iz0 += izPer) {
+    const int iz1 = min(iz0 + izPer, g.nz);
+    const int hb = cellStart[g.cellBase + iz0 * g.ny];
+    const int he = iz1 < g.nz ? cellStart[g.cellBase + iz1 * g.ny] : g.start + g.count;
+    const int bR = iz1 < g.nz ? z_bin(g.zmin + iz1 * g.cz - 1, g.zmin, z.zinv, z.nzb) : z.nzb - 1;
+    const int nb = min(bR - bL, kZBins);  // counters 1..nb for bins bL + 1..bR, counter 0 for the shared bin bL
+    for (int c = threadIdx.x; c <= nb; c += kZThreads) s_cnt[c] = 0;
+    __syncthreads();
+    for (int h = hb + threadIdx.x; h < he; h += kZThreads) {
+      const int b = z_bin(syz[h].y, g.zmin, z.zinv, z.nzb);
+      atomicAdd(&s_cnt[min(max(b - bL, 0), nb)], 1);
+    }
+    __syncthreads();
+    // exclusive scan of the nb + 1 counters: a run per thread
+    const int per = (nb + kZThreads) / kZThreads;
+    const int c0 = min(threadIdx.x * per, nb + 1), c1 = min(c0 + per, nb + 1);
+    int s = 0;
+    for (int c = c0; c < c1; ++c) s += s_cnt[c];
+    int x = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[w] = x;
+    __syncthreads();
+    int off = x - s;
+    for (int k = 0; k < w; ++k) off += s_warp[k];
+    const int base = hb - g.start;
+    for (int c = c0; c < c1; ++c) {
+      const int v = s_cnt[c];
+      s_cnt[c] = off;
+      if (c > 0) bins[bL + c] = base + off;
+      off += v;
+    }
+    __syncthreads();
+    for (int h = hb + threadIdx.x; h < he; h += kZThreads) {
+      const int2 p = syz[h];
+      const int b = z_bin(p.y, g.zmin, z.zinv, z.nzb);
+      const int pos = base + atomicAdd(&s_cnt[min(max(b - bL, 0), nb)], 1);
+      yz[pos] = p;
+      idx[pos] = h;
+    }
+    __syncthreads();
+    bL = bR;
+  }
+}
+
 // ------------------------------------------------------------- launchers
+void launch_zorder(int nRows, const RowGrid* grid, const int* rowMax, const int* cellStart, const int2* syz,
+                   ZRow* zrow, int4* bucket, cudaStream_t st) {
+  if (nRows > 0) {
+    k_zorder<<<nRows, kZThreads, 0, st>>>(grid, rowMax, cellStart, syz, zrow, bucket);
+    ++g_launch_count;
+  }
+}
+
 void launch_ingest_stats(const TFDesc* tfs, const int2* tiles, int nTiles, int tileSize, const GeomConst* G,
                          int* tileStats, unsigned* err, cudaStream_t st) {
   size_t smem = 3 * kRowsPerTF * sizeof(int);

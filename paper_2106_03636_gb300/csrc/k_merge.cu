@@ -442,9 +442,9 @@ __device__ int refit_chain(int head, int tail, const SectorTrackBufs& sb, const 
         const float dx = srow >= 0 ? (float)(ri - srow) * G->pitch : (float)(G->rowx_d[ri] - (double)t.x);
         if (kf_prop_dx_cov64(t, G->rowx_d[ri], dx, G->bzc) != 0) continue;
       } else if (srow >= 0) {
-        if (kf_prop_row<T>(t, srow, ri, G, bzc) != 0) continue;
+        if (kf_prop_row<T, kF1Rounded>(t, srow, ri, G, bzc) != 0) continue;
       } else {
-        if (kf_prop<T>(t, (T)G->rowx[ri], bzc) != 0) continue;
+        if (kf_prop<T, kF1Rounded>(t, (T)G->rowx[ri], bzc) != 0) continue;
       }
       srow = ri;
       recentre_y<T>(t.p[0], yref, p.x);

@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(128) k_tl_chain(const int* __restrict__ nTlDev
       const int row = r0 + (Rh - R0);
       const int2 hp = syz[hit];  // both loads in flight during the transport
       const int next = up[hit];
-      if (kf_prop_row<float>(st, prev, row, G, bzc) != 0) {
+      if (kf_prop_row<float, kF1Rounded>(st, prev, row, G, bzc) != 0) {
         dropped = true;
         break;
       }
@@ -184,13 +184,22 @@ __global__ void __launch_bounds__(128) k_tl_refit(const int* __restrict__ nTlDev
     const uint8_t* Rw = tb.rows + (size_t)k * kMaxTlHits;
     const int zref = tb.zref[k];
     int yref = tb.yref[k];
+    // from the top hit, with the direction that the outward pass left and a
+    // fresh covariance
     KState<float> st;
     float* S = tb.state + (size_t)k * 21;
-    load_state(st, S);
+    const int2 top = syz[H[na - 1]];
     int srow = Rw[na - 1];
+    st.x = G->rowx[srow];
+    st.p[0] = hit_y(top.x, yref);
+    st.p[1] = hit_z(top.y, zref, zunit);
+    st.p[2] = S[3];
+    st.p[3] = S[4];
+    st.p[4] = S[5];
+    reset_cov(st, G->angErr);
     for (int i = na - 2; i >= 0; --i) {
       const int2 hp = syz[H[i]];
-      if (kf_prop_row<float>(st, srow, Rw[i], G, bzc) != 0) continue;
+      if (kf_prop_row<float, kF1Rounded>(st, srow, Rw[i], G, bzc) != 0) continue;
       srow = Rw[i];
       recentre_y(st.p[0], yref, hp.x);
       kf_update<float>(st, hit_y(hp.x, yref), hit_z(hp.y, zref, zunit), nullptr, G->angErr);
@@ -213,9 +222,10 @@ __global__ void __launch_bounds__(128) k_tl_refit(const int* __restrict__ nTlDev
 // takes the next one (one atomic per warp for all such lanes), so the
 // transport and the update run converged whatever the tracklets' lengths.
 // The row search comes in two forms that pick the same hit:
-// * per lane: each lane scans the candidate cells of its own window;
-// * warp-cooperative: the candidates of all lanes' windows on this step are
-//   laid out one after another and scanned 32 at a time by the whole warp
+// * per lane: each lane scans the candidates of its own window, in the row's
+//   drift-ordered view;
+// * warp-cooperative: the candidate cells of all lanes' windows on this step
+//   are laid out one after another and scanned 32 at a time by the whole warp
 //   (a lane finds the owner of candidate q by a binary search over the
 //   warp's exclusive candidate offsets; per owner the smallest key wins).
 // Both score a candidate by the same explicitly rounded expression and keep
@@ -228,23 +238,18 @@ struct SearchPar {
   int yref, zref;
 };
 
-// Window of a row search; false: no candidate can pass (empty row, unusable
-// window).  The cell rectangle only has to cover the window: one unit of
+// Window of a row search: its parameters and drift range; false: unusable, no
+// candidate can pass.  The range only has to cover the window: one unit of
 // slack on each side absorbs the rounding of the float products.
-__device__ inline bool search_window(const RowGrid& g, int npads, const KState<float>& s, int yref, int zref,
-                                     float izunit, int angErr, SearchPar& P, int& iy0, int& iy1, int& iz0,
-                                     int& iz1) {
-  if (g.count == 0) return false;
+__device__ inline bool search_window(const KState<float>& s, int yref, int zref, float izunit, int angErr,
+                                     SearchPar& P, int& zlo, int& zhi) {
   float vy, vz;
   meas_var<float>(angErr, s, vy, vz);
   const float sy2 = s.C[0] + vy, sz2 = s.C[2] + vz;
   const float wy = 3.f * sqrtf(sy2), wz = 3.f * sqrtf(sz2);
   if (!(wy < 1e4f) || !(wz < 1e4f) || !isfinite(s.p[0]) || !isfinite(s.p[1])) return false;
-  const int ylo = yref + clamp_i(floorf((s.p[0] - wy) * 160.f)) - 1;
-  const int yhi = yref + clamp_i(ceilf((s.p[0] + wy) * 160.f)) + 1;
-  const int zlo = zref + clamp_i(floorf((s.p[1] - wz) * izunit)) - 1;
-  const int zhi = zref + clamp_i(ceilf((s.p[1] + wz) * izunit)) + 1;
-  if (!cell_range(g, npads, ylo, yhi, zlo, zhi, iy0, iy1, iz0, iz1)) return false;
+  zlo = zref + clamp_i(floorf((s.p[1] - wz) * izunit)) - 1;
+  zhi = zref + clamp_i(ceilf((s.p[1] + wz) * izunit)) + 1;
   P.y = s.p[0];
   P.z = s.p[1];
   P.wy = wy;
@@ -254,6 +259,11 @@ __device__ inline bool search_window(const RowGrid& g, int npads, const KState<f
   P.yref = yref;
   P.zref = zref;
   return true;
+}
+// The window's y range in units, with the same slack.
+__device__ inline void window_y(const SearchPar& P, int& ylo, int& yhi) {
+  ylo = P.yref + clamp_i(floorf((P.y - P.wy) * 160.f)) - 1;
+  yhi = P.yref + clamp_i(ceilf((P.y + P.wy) * 160.f)) + 1;
 }
 
 constexpr unsigned long long kNoHit = ~0ull;
@@ -270,21 +280,67 @@ __device__ inline unsigned long long cand_key(int h, int2 p, const SearchPar& P,
   return ((unsigned long long)__float_as_uint(chi) << 32) | (unsigned)h;
 }
 
-// Per-lane search: cell rows [iz0, iz0 + nseg) x columns [iy0, iy1].
-__device__ inline unsigned long long lane_search(int nseg, int cellBase, int ny, int iy0, int iy1, int iz0,
-                                                 const int* __restrict__ cellStart, const int2* __restrict__ syz,
-                                                 const SearchPar& P, float zunit) {
+// Best hit of a search: its sorted index (-1: none) and coordinates.
+struct BestHit {
+  int hit;
+  int2 p;
+};
+
+// Per-lane search through the cells [iy0, iy1] of rows [iz0, iz1] (rows so
+// dense that the cells hold fewer candidates than the drift window).
+__device__ inline BestHit cell_search(const RowGrid& g, int iy0, int iy1, int iz0, int iz1,
+                                      const int* __restrict__ cellStart, const int2* __restrict__ syz,
+                                      const SearchPar& P, float zunit) {
   unsigned long long best = kNoHit;
-  for (int j = 0; j < nseg; ++j) {
-    const int cb = cellBase + (iz0 + j) * ny;
+  BestHit B{-1, make_int2(0, 0)};
+  for (int iz = iz0; iz <= iz1; ++iz) {
+    const int cb = g.cellBase + iz * g.ny;
     const int a = __ldg(cellStart + cb + iy0);
     const int b = __ldg(cellStart + cb + iy1 + 1);
     for (int h = a; h < b; ++h) {
-      const unsigned long long key = cand_key(h, __ldg(syz + h), P, zunit);
-      if (key < best) best = key;
+      const int2 p = __ldg(syz + h);
+      const unsigned long long key = cand_key(h, p, P, zunit);
+      if (key < best) {
+        best = key;
+        B.hit = h;
+        B.p = p;
+      }
     }
   }
-  return best;
+  return B;
+}
+
+// Per-lane search through positions [a, b) of a row's drift-ordered view:
+// four candidates loaded at once (a window holds 3-4 on average), so a row
+// step waits for one load and not for one per candidate.  Equal chi2 goes to
+// the smaller sorted index.
+__device__ inline BestHit z_search(const ZView& V, const ZRow& g, int a, int b, const SearchPar& P, float zunit) {
+  const int2* yz = V.yz(g);
+  const int* idx = V.idx(g);
+  unsigned best = ~0u;
+  int pos = -1;
+  BestHit B{-1, make_int2(0, 0)};
+  for (int h = a; h < b; h += 4) {
+    int2 q[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) q[u] = __ldg(yz + min(h + u, b - 1));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const unsigned long long key = cand_key(0, q[u], P, zunit);
+      const unsigned c = (unsigned)(key >> 32);
+      if (key != kNoHit && h + u < b) {
+        bool take = c < best;
+        if (c == best) take = __ldg(idx + h + u) < __ldg(idx + pos);
+        if (take) {
+          best = c;
+          pos = h + u;
+          B.p = q[u];
+        }
+      }
+    }
+  }
+  if (pos >= 0) B.hit = __ldg(idx + pos);
+  return B;
 }
 
 // Warp-cooperative search.  Lane l searches cell rows [iz0, iz0 + nseg) x
@@ -350,23 +406,17 @@ __device__ inline unsigned long long coop_search(int nseg, int cellBase, int ny,
 }
 
 // (b) kDir = +1: outward following above the chain; its result is the
-// inward refit's starting state: the last accepted state with the position
-// of the top hit and a fresh covariance.  (d) kDir = -1: inward following
-// below the chain start; the state kept is the one at the innermost accepted
-// hit.  coop: 1 warp-cooperative search, 0 per-lane search.
-// Blocks of 128 per SM the following kernels are compiled for: 7 (72
-// registers, no spills) measured 2 % faster over both passes on the full
-// Time Frame than 8 (64 registers, ~40 bytes of spills).
-#ifndef O2TPC_FOLLOW_MIN_BLOCKS
-#define O2TPC_FOLLOW_MIN_BLOCKS 7
-#endif
-
+// inward refit's starting point: the direction parameters of the last
+// accepted state (position: the top hit; fresh covariance).  (d) kDir = -1:
+// inward following below the chain start; the state kept is the one at the
+// innermost accepted hit.
+// This form searches warp-cooperatively (O2TPC_FLAG_COOP_SEARCH).
 template <int kDir>
-__global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS) k_tl_follow(const int* __restrict__ nTlDev, int* __restrict__ counter,
+__global__ void __launch_bounds__(128, 7) k_tl_follow_coop(const int* __restrict__ nTlDev, int* __restrict__ counter,
                                                      const RowGrid* __restrict__ grid,
                                                      const int* __restrict__ cellStart,
                                                      const int2* __restrict__ syz,
-                                                     const GeomConst* __restrict__ G, TrackletBufs tb, int coop) {
+                                                     const GeomConst* __restrict__ G, TrackletBufs tb) {
   __shared__ float s_last[21][128];
   __shared__ SearchPar s_par[128];
   __shared__ unsigned long long s_best[128];
@@ -446,26 +496,24 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS) k_tl_follow(cons
     if (have) {
       if ((kDir > 0) ? (r >= kNRow) : (r < 0)) {
         finish();
-      } else if (kf_prop_row<float>(st, srow, r, G, bzc) != 0 || fabsf(st.p[2]) > kSinFollow) {
+      } else if (kf_prop_row<float, kF1Fused>(st, srow, r, G, bzc) != 0 || fabsf(st.p[2]) > kSinFollow) {
         finish();
       } else {
         srow = r;
         const RowGrid g = grid[Rs + r];
-        if (search_window(g, G->npads[r], st, yref, zref, izunit, G->angErr, P, iy0, iy1, iz0, iz1)) {
-          nseg = iz1 - iz0 + 1;
+        int ylo, yhi, zlo, zhi;
+        if (g.count > 0 && search_window(st, yref, zref, izunit, G->angErr, P, zlo, zhi)) {
+          window_y(P, ylo, yhi);
+          if (cell_range(g, G->npads[r], ylo, yhi, zlo, zhi, iy0, iy1, iz0, iz1)) nseg = iz1 - iz0 + 1;
           cellBase = g.cellBase;
           ny = g.ny;
         }
       }
     }
-    unsigned long long best;
-    if (coop) {
-      if (nseg > 0) s_par[threadIdx.x] = P;
-      __syncwarp();
-      best = coop_search(nseg, cellBase, ny, iy0, iy1, iz0, cellStart, syz, s_par + wb, s_best + wb, zunit);
-    } else {
-      best = lane_search(nseg, cellBase, ny, iy0, iy1, iz0, cellStart, syz, P, zunit);
-    }
+    if (nseg > 0) s_par[threadIdx.x] = P;
+    __syncwarp();
+    const unsigned long long best =
+        coop_search(nseg, cellBase, ny, iy0, iy1, iz0, cellStart, syz, s_par + wb, s_best + wb, zunit);
     if (have) {
       if (best != kNoHit) {
         const int hit = (int)(unsigned)(best & 0xffffffffull);
@@ -477,6 +525,144 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS) k_tl_follow(cons
         ++n;
         save_last(st);
         yrefLast = yref;
+        misses = 0;
+        r += kDir;
+      } else if (++misses >= kMaxMiss) {
+        finish();
+      } else {
+        r += kDir;
+      }
+    }
+  }
+}
+
+// The same passes with the per-lane search in the drift-ordered views (rows
+// flagged dense: in the cells).  Bound by the latency of the dependent chain of a row
+// step (row table -> bin starts -> candidates -> update) and by its ~450
+// instructions.  Only what the next reader needs survives a step: the
+// direction parameters and the row of the last accepted state (with kKeep the
+// whole state, for inspection), so nothing is copied per accepted hit.
+// Measured against the search in the cells with the state copied per hit:
+// 1 ms frame (20.3 M clusters) 2.26 + 1.73 -> 1.66 + 1.40 ms, 32 orbits (59 M)
+// 6.87 + 5.19 -> 4.98 + 4.12 ms, 3 collisions (1.3 M, one tracklet a lane)
+// 0.58 + 0.55 -> 0.43 + 0.48 ms.
+// Blocks of 128 per SM the kernel is compiled for:
+#ifndef O2TPC_FOLLOW_MIN_BLOCKS
+#define O2TPC_FOLLOW_MIN_BLOCKS 7
+#endif
+
+template <int kDir, bool kKeep>
+__global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
+    k_tl_follow(const int* __restrict__ nTlDev, int* __restrict__ counter, const RowGrid* __restrict__ grid,
+                const int* __restrict__ cellStart, const int2* __restrict__ syz, const GeomConst* __restrict__ G,
+                ZView zv, TrackletBufs tb) {
+  constexpr bool kWhole = kKeep && kDir < 0;
+  __shared__ float s_last[kWhole ? 20 : 1][128];
+  const unsigned full = 0xffffffffu;
+  const float zunit = G->zunit, izunit = G->kz, bzc = G->bzc;
+  const int angErr = G->angErr;
+  const int nTl = *nTlDev;
+  bool have = false, exhausted = false;
+  int k = 0, r = 0, n = 0, misses = 0, srow = 0, yref = 0, yrefLast = 0, zref = 0, Rs = 0, lastRow = 0;
+  float last2 = 0.f, last3 = 0.f, last4 = 0.f;
+  KState<float> st;
+  auto save_last = [&]() {
+    last2 = st.p[2];
+    last3 = st.p[3];
+    last4 = st.p[4];
+    lastRow = srow;
+    yrefLast = yref;
+    if (kWhole) {
+#pragma unroll
+      for (int j = 0; j < 5; ++j) s_last[j % (kWhole ? 20 : 1)][threadIdx.x] = st.p[j];
+#pragma unroll
+      for (int j = 0; j < 15; ++j) s_last[(5 + j) % (kWhole ? 20 : 1)][threadIdx.x] = st.C[j];
+    }
+  };
+  // ends the lane's tracklet with the state after its last accepted hit
+  auto finish = [&]() {
+    float* S = tb.state + (size_t)k * 21;
+    if (kDir > 0) {
+      tb.nasc[k] = n;
+      tb.yref[k] = yrefLast;
+    } else {
+      tb.nhits[k] = n;
+      S[0] = G->rowx[lastRow];
+    }
+    S[3] = last2;
+    S[4] = last3;
+    S[5] = last4;
+    if (kWhole) {
+      S[1] = s_last[0][threadIdx.x] + (float)yrefLast * 0.00625f;
+      S[2] = s_last[1 % (kWhole ? 20 : 1)][threadIdx.x];
+#pragma unroll
+      for (int j = 0; j < 15; ++j) S[6 + j] = s_last[(5 + j) % (kWhole ? 20 : 1)][threadIdx.x];
+    }
+    have = false;
+  };
+  for (;;) {
+    // lanes without a tracklet take the next ones
+    const bool want = !have && !exhausted;
+    const int kk = warp_take(counter, want);
+    if (want) {
+      k = kk;
+      if (k >= nTl) {
+        exhausted = true;
+      } else {
+        const int na = tb.nasc[k];
+        if (na > 0) {
+          const uint8_t* Rw = tb.rows + (size_t)k * kMaxTlHits;
+          Rs = tb.rbase[k];
+          zref = tb.zref[k];
+          yref = tb.yref[k];
+          load_state(st, tb.state + (size_t)k * 21);
+          n = na;
+          r = (kDir > 0) ? Rw[na - 1] + 1 : Rw[0] - 1;
+          misses = 0;
+          srow = row_of_x(st.x);
+          save_last();
+          have = true;
+        }
+      }
+    }
+    if (__ballot_sync(full, have) == 0) {
+      if (__all_sync(full, exhausted)) break;
+      continue;
+    }
+    // one row step of every busy lane: transport, then the window
+    BestHit best{-1, make_int2(0, 0)};
+    if (have) {
+      if ((kDir > 0) ? (r >= kNRow) : (r < 0)) {
+        finish();
+      } else if (kf_prop_row<float, kF1Fused>(st, srow, r, G, bzc) != 0 || fabsf(st.p[2]) > kSinFollow) {
+        finish();
+      } else {
+        srow = r;
+        const ZRow g = zv.rows[Rs + r];
+        SearchPar P;
+        int zlo, zhi;
+        if (g.count > 0 && search_window(st, yref, zref, izunit, angErr, P, zlo, zhi)) {
+          if (g.flags & kZFollowCells) {
+            const RowGrid gc = grid[Rs + r];
+            int ylo, yhi, iy0, iy1, iz0, iz1;
+            window_y(P, ylo, yhi);
+            if (cell_range(gc, G->npads[r], ylo, yhi, zlo, zhi, iy0, iy1, iz0, iz1))
+              best = cell_search(gc, iy0, iy1, iz0, iz1, cellStart, syz, P, zunit);
+          } else {
+            int a, b;
+            if (z_range(zv, g, zlo, zhi, a, b)) best = z_search(zv, g, a, b, P, zunit);
+          }
+        }
+      }
+    }
+    if (have) {
+      if (best.hit >= 0) {
+        recentre_y(st.p[0], yref, best.p.x);
+        kf_update<float>(st, hit_y(best.p.x, yref), hit_z(best.p.y, zref, zunit), nullptr, angErr);
+        tb.hits[(size_t)k * kMaxTlHits + n] = best.hit;
+        tb.rows[(size_t)k * kMaxTlHits + n] = (uint8_t)r;
+        ++n;
+        save_last();
         misses = 0;
         r += kDir;
       } else if (++misses >= kMaxMiss) {
@@ -732,7 +918,7 @@ __global__ void __launch_bounds__(128) k_sector_fit(const int* __restrict__ nStD
   kf_meas_cov<float>(t, G->angErr);
   int srow = Rw[0], zcur = zref;
   for (int i = 1; i < m; ++i) {
-    if (kf_prop_row<float>(t, srow, Rw[i], G, bzc) != 0) continue;
+    if (kf_prop_row<float, kF1Fused>(t, srow, Rw[i], G, bzc) != 0) continue;
     srow = Rw[i];
     p = P[i];
     recentre_y(t.p[0], yref, p.x);
@@ -750,7 +936,7 @@ __global__ void __launch_bounds__(128) k_sector_fit(const int* __restrict__ nStD
   zcur = P[m - 1].y;
   u.p[1] = 0.f;
   for (int i = m - 2; i >= 0; --i) {
-    if (kf_prop_row<float>(u, srow, Rw[i], G, bzc) != 0) continue;
+    if (kf_prop_row<float, kF1Rounded>(u, srow, Rw[i], G, bzc) != 0) continue;
     srow = Rw[i];
     p = P[i];
     recentre_y(u.p[0], yref, p.x);
@@ -773,9 +959,9 @@ PassGrid pass_grid() {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&g.sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g.chain, k_tl_chain, 128, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g.out, k_tl_follow<1>, 128, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g.out, k_tl_follow<1, false>, 128, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g.refit, k_tl_refit, 128, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g.in, k_tl_follow<-1>, 128, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g.in, k_tl_follow<-1, false>, 128, 0);
   }
   return g;
 }
@@ -783,7 +969,8 @@ PassGrid pass_grid() {
 
 void launch_tracklets(int nTl, const int* nTlDev, int* workCounter, const int* starts, const int* up,
                       const RowGrid* grid, int nRows, const int* cellStart, const int2* syz, const GeomConst* G,
-                      TrackletBufs tb, cudaStream_t st, cudaEvent_t* passEnd, bool coopSearch) {
+                      ZView zv, TrackletBufs tb, cudaStream_t st, cudaEvent_t* passEnd, bool coopSearch,
+                      bool keepState) {
   auto mark = [&](int i) {
     if (passEnd) cudaEventRecord(passEnd[i], st);
   };
@@ -796,12 +983,19 @@ void launch_tracklets(int nTl, const int* nTlDev, int* workCounter, const int* s
   cudaMemsetAsync(workCounter, 0, 4 * sizeof(int), st);
   k_tl_chain<<<blocks(g.chain), 128, 0, st>>>(nTlDev, workCounter, starts, up, grid, nRows, syz, G, tb);
   mark(0);
-  const int coop = coopSearch ? 1 : 0;
-  k_tl_follow<1><<<blocks(g.out), 128, 0, st>>>(nTlDev, workCounter + 1, grid, cellStart, syz, G, tb, coop);
+  if (coopSearch)
+    k_tl_follow_coop<1><<<blocks(g.out), 128, 0, st>>>(nTlDev, workCounter + 1, grid, cellStart, syz, G, tb);
+  else
+    k_tl_follow<1, false><<<blocks(g.out), 128, 0, st>>>(nTlDev, workCounter + 1, grid, cellStart, syz, G, zv, tb);
   mark(1);
   k_tl_refit<<<blocks(g.refit), 128, 0, st>>>(nTlDev, workCounter + 2, syz, G, tb);
   mark(2);
-  k_tl_follow<-1><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, grid, cellStart, syz, G, tb, coop);
+  if (coopSearch)
+    k_tl_follow_coop<-1><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, grid, cellStart, syz, G, tb);
+  else if (keepState)
+    k_tl_follow<-1, true><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, grid, cellStart, syz, G, zv, tb);
+  else
+    k_tl_follow<-1, false><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, grid, cellStart, syz, G, zv, tb);
   mark(3);
   g_launch_count += 4;
 }

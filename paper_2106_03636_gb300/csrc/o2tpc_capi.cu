@@ -685,6 +685,10 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
     autotune(c, n, nRows, rowCnt, rowMin, rowMax, grid, nfBlockStart, totals, bucket, cellStart, syz, sorig, gscratch,
              dErr);
   CKL();
+  ZRow* zrow = dalloc<ZRow>(M, nRows);
+  launch_zorder(nRows, grid, rowMax, cellStart, syz, zrow, bucket, st);
+  CKL();
+  const ZView zv{zrow, reinterpret_cast<const char*>(bucket)};
 
   // ---- A5-A7: neighbours, cleaner, start hits
   CK(cudaEventRecord(c->evs[2], st));
@@ -731,8 +735,8 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   tb.yref = dalloc<int>(M, nTl);
   tb.rbase = dalloc<int>(M, nTl);
   int* workCounter = dalloc<int>(M, 4);
-  launch_tracklets(nTl, &C->nTl, workCounter, starts, up, grid, nRows, cellStart, syz, G, tb, st, c->evTl,
-                   (c->cfg.flags & O2TPC_FLAG_COOP_SEARCH) != 0);
+  launch_tracklets(nTl, &C->nTl, workCounter, starts, up, grid, nRows, cellStart, syz, G, zv, tb, st, c->evTl,
+                   (c->cfg.flags & O2TPC_FLAG_COOP_SEARCH) != 0, (c->cfg.flags & O2TPC_FLAG_KEEP_STAGES) != 0);
   CKL();
 
   // ---- A9: selection

@@ -67,6 +67,7 @@ size_t graph_carve(GraphArena& A, char* base) {
   take(A.cellStart, k.cellsCap + 1);
   take(A.gscratch, k.cellsCap);
   take(A.bucket, n);
+  take(A.zrow, k.nRows);
   take(A.syz, n + 2);
   take(A.sorig, n);
   take(A.upRaw, n);
@@ -177,6 +178,8 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   launch_grid(k.nRows, A.rowCnt, A.rowMin, A.rowMax, G, A.grid, A.nfBlockStart, nfBlock, A.totals, st);
   launch_row_scatter(A.tfs, A.tiles, k.nTilesCap, k.tileSize, G, A.tileStats, A.grid, A.bucket, st);
   launch_cell_sort(k.nRows, A.grid, A.bucket, A.cellStart, A.syz, A.sorig, A.gscratch, A.totals, st, sortThreads);
+  launch_zorder(k.nRows, A.grid, A.rowMax, A.cellStart, A.syz, A.zrow, A.bucket, st);
+  const ZView zv{A.zrow, reinterpret_cast<const char*>(A.bucket)};
   // A5-A7
   launch_neighbours(n / nfBlock + k.nRows + 1, nfBlock, nfStage, A.grid, A.nfBlockStart, k.nRows, A.cellStart, A.syz, G,
                     A.upRaw, A.dnRaw, A.err, st);
@@ -186,8 +189,8 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   launch_ballot_compact(n, &C->n, A.flag, A.tileOff, A.starts, k.tlCap, &C->overflow, st);
   launch_tf_ranges(k.BCap, A.grid, A.starts, &C->nTl, A.tlTfBegin, st);
   // A8
-  launch_tracklets(k.tlCap, &C->nTl, A.workCounter, A.starts, A.up, A.grid, k.nRows, A.cellStart, A.syz, G, A.tb,
-                   st, nullptr, coopSearch);
+  launch_tracklets(k.tlCap, &C->nTl, A.workCounter, A.starts, A.up, A.grid, k.nRows, A.cellStart, A.syz, G, zv,
+                   A.tb, st, nullptr, coopSearch);
   // A9
   cudaMemsetAsync(A.w, 0, sizeof(unsigned long long) * (size_t)n, st);
   launch_ownership(k.tlCap, &C->nTl, k.BCap * kNSec, A.grid, A.starts, A.tb, A.w, A.secBegin, A.wide, st);

@@ -30,7 +30,8 @@ struct GraphArena {
   int* totals;
   int* cellStart;
   int* gscratch;
-  int4* bucket;
+  int4* bucket;  // row buckets of the sort, then the drift-ordered views
+  ZRow* zrow;
   int2* syz;
   int* sorig;
   int *upRaw, *dnRaw, *up, *dn, *flag, *tileCnt, *tileOff, *scratch;

@@ -73,6 +73,60 @@ struct RowGrid {
   int pad;
 };
 
+// Drift-ordered view of a row, 32 bytes.  The row's hits once more, ordered by
+// drift bin (any order inside a bin): the searches around a predicted point
+// look through the bins their drift window touches.  A window of 1-4 cm
+// holds 2-8 hits of a whole pad row at 50 kHz Pb-Pb, where the cells of the
+// sorted order (2 cm x 40-110 cm there: 4 hits each) that cover the same
+// window hold 10 or more.  The view lives in the row's bucket records, which
+// the cell sort has used up (16 bytes per hit: coordinates 8, sorted index 4,
+// bin starts 4 - so a row has at most as many bins as hits).
+struct ZRow {
+  int start;    // first sorted hit of the row (batch-global), as RowGrid
+  int count;
+  int zmin;
+  int nzb;      // drift bins
+  float zinv;   // bins per drift unit
+  int flags;    // kZNFCells, kZFollowCells
+  int pad0, pad1;
+};
+// Rows so dense that the cells hold fewer candidates than the drift window:
+// bit 0 for the NeighboursFinder's window, bit 1 for the following's.
+enum : int { kZNFCells = 1, kZFollowCells = 2 };
+
+// The drift-ordered views of a batch: row tables and the record memory.
+struct ZView {
+  const ZRow* rows;
+  const char* mem;
+  __device__ const int2* yz(const ZRow& g) const { return reinterpret_cast<const int2*>(mem + 16ll * g.start); }
+  __device__ const int* idx(const ZRow& g) const {
+    return reinterpret_cast<const int*>(mem + 16ll * g.start + 8ll * g.count);
+  }
+  __device__ const int* bins(const ZRow& g) const {
+    return reinterpret_cast<const int*>(mem + 16ll * g.start + 12ll * g.count);
+  }
+};
+
+// Drift bin of a coordinate at or above the row's zmin.  Conversion and
+// product round monotonically, so the bins are ordered like the coordinates:
+// the hits of a window [zlo, zhi] lie in the bins of its ends or between.
+__host__ __device__ inline int z_bin(int z, int zmin, float zinv, int nzb) {
+  const int b = (int)((float)((unsigned)z - (unsigned)zmin) * zinv);
+  return b < nzb - 1 ? b : nzb - 1;
+}
+
+// Positions [a, b) of the row's view that hold every hit with a drift
+// coordinate in [zlo, zhi]; false if there is none.
+__device__ inline bool z_range(const ZView& V, const ZRow& g, int zlo, int zhi, int& a, int& b) {
+  if (g.count == 0 || zhi < g.zmin) return false;
+  const int b0 = zlo <= g.zmin ? 0 : z_bin(zlo, g.zmin, g.zinv, g.nzb);
+  const int b1 = z_bin(zhi, g.zmin, g.zinv, g.nzb);
+  const int* zs = V.bins(g);
+  a = __ldg(zs + b0);
+  b = b1 + 1 < g.nzb ? __ldg(zs + b1 + 1) : g.count;
+  return a < b;
+}
+
 // Per-TF descriptor of a batch.
 struct TFDesc {
   const void* in0;   // FLOAT: sector (uint8) / FIXED: packed records
@@ -284,7 +338,12 @@ template <typename T>
 struct PropStep {
   T dy, dzeta, s2, a02, a04, a12, a13, a14, a24;
 };
-template <typename T>
+// kF1: f1 + 4 fm can be rounded two ways in single precision - from f1
+// itself, or fused with the last product of f1 (the difference reaches the
+// covariance's y-zeta terms in the last place).  The compiler picks one by
+// what surrounds the call; a caller that must not depend on that names it.
+enum : int { kF1Any = 0, kF1Rounded = 1, kF1Fused = 2 };
+template <typename T, int kF1 = kF1Any>
 __device__ inline int kf_prop_step(const T* p, T dx, T bzc, PropStep<T>& o) {
   T s1 = p[2], q = p[4], tz = p[3];
   T k = q * bzc;
@@ -317,7 +376,14 @@ __device__ inline int kf_prop_step(const T* p, T dx, T bzc, PropStep<T>& o) {
   T cm = kf_sqrt<T>((T(1) - sm) * (T(1) + sm));
   T f1 = dx * (s1 + s2) * ic1 * ic2 * icc;
   T fm = T(0.5) * dx * (sm + s2) * ic2 / (cm * (cm + c2));
-  T ddsdk = (fabs(k * dx) < T(0.05)) ? dx * (f1 + T(4) * fm) * T(1.0 / 6.0) : (dx * ic2 - ds) / k;
+  T ddsdk;
+  if constexpr (kF1 == kF1Any) {
+    ddsdk = (fabs(k * dx) < T(0.05)) ? dx * (f1 + T(4) * fm) * T(1.0 / 6.0) : (dx * ic2 - ds) / k;
+  } else {
+    const float sum =
+        kF1 == kF1Rounded ? __fmaf_rn(4.f, fm, f1) : __fmaf_rn(dx * (s1 + s2) * ic1 * ic2, icc, 4.f * fm);
+    ddsdk = (fabs(k * dx) < T(0.05)) ? dx * sum * T(1.0 / 6.0) : (dx * ic2 - ds) / k;
+  }
   const T a02 = dx * (T(2) * cc + (s1 + s2) * (s1 * ic1 + s2 * ic2)) * icc * icc;
   const T a04 = dx * dx * bzc * (cc + (s1 + s2) * s2 * ic2) * icc * icc;
   const T a12 = tz * f1;
@@ -336,11 +402,11 @@ __device__ inline int kf_prop_step(const T* p, T dx, T bzc, PropStep<T>& o) {
   return 0;
 }
 
-template <typename T>
+template <typename T, int kF1 = kF1Any>
 __device__ inline int kf_prop_dx(KState<T>& s, T x2, T dx, T bzc) {
   if (dx == T(0)) return 0;
   PropStep<T> o;
-  if (kf_prop_step<T>(s.p, dx, bzc, o) != 0) return -1;
+  if (kf_prop_step<T, kF1>(s.p, dx, bzc, o) != 0) return -1;
   s.p[0] += o.dy;
   s.p[1] += o.dzeta;
   s.p[2] = o.s2;
@@ -372,9 +438,9 @@ __device__ inline int kf_prop_dx_cov64(KState<double>& s, double x2, float dx, f
 
 // Transport to x2 from a state at any x (after a frame rotation, or to another
 // track's x): the step is the difference of the two positions.
-template <typename T>
+template <typename T, int kF1 = kF1Any>
 __device__ inline int kf_prop(KState<T>& s, T x2, T bzc) {
-  return kf_prop_dx<T>(s, x2, x2 - s.x, bzc);
+  return kf_prop_dx<T, kF1>(s, x2, x2 - s.x, bzc);
 }
 
 // Transport between pad rows r1 -> r2 of a state sitting on row r1.  The step
@@ -382,11 +448,11 @@ __device__ inline int kf_prop(KState<T>& s, T x2, T bzc) {
 // row positions would carry up to 1.5e-5 cm in single precision, an error
 // that dominates the FP32 curvature of short tracks (a 10-row stub's
 // sagitta is a few 1e-3 cm).
-template <typename T>
+template <typename T, int kF1 = kF1Any>
 __device__ inline int kf_prop_row(KState<T>& s, int r1, int r2, const GeomConst* __restrict__ G, T bzc) {
   const T pitch = sizeof(T) == 8 ? (T)G->pitch_d : (T)G->pitch;
   const T x2 = sizeof(T) == 8 ? (T)G->rowx_d[r2] : (T)G->rowx[r2];
-  return kf_prop_dx<T>(s, x2, (T)(r2 - r1) * pitch, bzc);
+  return kf_prop_dx<T, kF1>(s, x2, (T)(r2 - r1) * pitch, bzc);
 }
 
 // Pad row of a state whose x is a row position (within its rounding).

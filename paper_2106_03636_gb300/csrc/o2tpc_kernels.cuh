@@ -27,6 +27,11 @@ void launch_cell_sort(int nRows, const RowGrid* grid, const int4* bucket, int* c
                       int* gscratch, const int* totals, cudaStream_t st,
                       int threadsPerRow = 256);
 
+// The drift-ordered views (ZRow) of all rows, written over the bucket records
+// of the rows (used up by the cell sort; their memory stays the view's).
+void launch_zorder(int nRows, const RowGrid* grid, const int* rowMax, const int* cellStart, const int2* syz,
+                   ZRow* zrow, int4* bucket, cudaStream_t st);
+
 // k_ca.cu
 // syz must hold one int2 of padding past the last hit (the 16-byte aligned
 // slab copies may read it); err collects kErrTimeout.  inject: the context's
@@ -90,18 +95,22 @@ struct TrackletBufs {
   int* nasc;     // [nTl]  hits in slots [0, nasc) in ascending rows; slots [nasc, nhits) descending
   int* hits;     // [nTl * kMaxTlHits]
   uint8_t* rows; // [nTl * kMaxTlHits]
-  float* state;  // [nTl * 21]  x, par[5], cov[15] at the innermost hit
+  float* state;  // [nTl * 21]  x, par[5], cov[15] at the innermost hit (x, par[2..4] without keepState)
   int* zref;     // [nTl]
   int* yref;     // [nTl]  y origin (units) of the state handed between the passes
   int* rbase;    // [nTl]  batch-global row of pad row 0 of the tracklet's sector
 };
 // passEnd: optional 4 events recorded after the chain-fit, outward, refit and
 // inward passes.  coopSearch: the following passes scan the row windows
-// cooperatively over the warp instead of lane by lane (identical results).
+// cooperatively over the warp, in the cells, instead of lane by lane in the
+// drift-ordered views (identical results).  keepState: leave the whole state
+// in tb.state; without it the inward pass leaves x and the three direction
+// parameters, which is all the sector fits read.
 // nTl sizes the grids; the kernels read the count at nTlDev
 void launch_tracklets(int nTl, const int* nTlDev, int* workCounter, const int* starts, const int* up,
                       const RowGrid* grid, int nRows, const int* cellStart, const int2* syz, const GeomConst* G,
-                      TrackletBufs tb, cudaStream_t st, cudaEvent_t* passEnd = nullptr, bool coopSearch = false);
+                      ZView zv, TrackletBufs tb, cudaStream_t st, cudaEvent_t* passEnd = nullptr,
+                      bool coopSearch = false, bool keepState = false);
 
 struct SectorTrackBufs {
   int* tl;        // [nSt] tracklet of the sector track
