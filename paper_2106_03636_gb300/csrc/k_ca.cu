@@ -54,9 +54,247 @@ __device__ inline int nf_collect(const RowGrid& g, int iy0, int iy1, int iz0, in
   return n;
 }
 
-// K4: one thread per hit; blocks of kB hits tile the rows
-// (nfBlockStart, built for the same block size, maps a block to its row,
-// looked up once per block).
+// One hit's best pair in the cell rectangles of the adjacent rows; su / sd:
+// coordinates of sorted hit c at su[c - bu0] / sd[c - bd0] (a staged slab, or
+// the global array with offset 0).
+__device__ inline void nf_cells(const RowGrid& gu, const RowGrid& gd, int uy0, int uy1, int uz0, int uz1, int dy0,
+                                int dy1, int dz0, int dz1, const int* __restrict__ cellStart,
+                                const int2* __restrict__ syz, const int2* su, int bu0, const int2* sd, int bd0, int2 hh,
+                                int& bu, int& bd) {
+  const int yh = hh.x, zh = hh.y;
+  int ui[kNFCand] = {}, di[kNFCand] = {};
+  unsigned ur[kNFCand] = {}, dr[kNFCand] = {};
+  const int nu = nf_collect(gu, uy0, uy1, uz0, uz1, cellStart, su, bu0, hh, ui, ur);
+  const int nd = nu > 0 ? nf_collect(gd, dy0, dy1, dz0, dz1, cellStart, sd, bd0, hh, di, dr) : 0;
+  // bestD starts one above the cut, so "D < bestD" also applies the cut
+  int bestD = kMaxMetric + 1;
+  // pairs in ascending (u, d): a strict "<" keeps the first minimum,
+  // which is the lexicographic minimum of (D, u, d).  Slots [a0, kNFCand)
+  // of both sides: the last four when both sides fit there (the common
+  // case), else all of them.
+  auto pair_scan = [&](const int a0) {
+#pragma unroll
+    for (int a = a0; a < kNFCand; ++a)
+#pragma unroll
+      for (int b = a0; b < kNFCand; ++b) {
+        const unsigned sres = ur[a] + dr[b];
+        const int ey = (int)(sres >> 16) - 2048, ez = (int)(sres & 0xFFFFu) - 2048;
+        const int D = kWeightY * ey * ey + kWeightZ * ez * ez;
+        if (a >= kNFCand - nu && b >= kNFCand - nd && D < bestD) {
+          bestD = D;
+          bu = ui[a];
+          bd = di[b];
+        }
+      }
+  };
+  constexpr int kNFSmall = kNFCand < 4 ? kNFCand : 4;
+  if (nu <= kNFSmall && nd <= kNFSmall) {
+    pair_scan(kNFCand - kNFSmall);
+  } else if (nu <= kNFCand && nd <= kNFCand) {
+    pair_scan(0);
+  } else {
+    const int y2 = 2 * yh, z2 = 2 * zh;
+    for (int izu = uz0; izu <= uz1; ++izu) {
+      const int ua = __ldg(cellStart + gu.cellBase + izu * gu.ny + uy0);
+      const int ub = __ldg(cellStart + gu.cellBase + izu * gu.ny + uy1 + 1);
+      for (int u = ua; u < ub; ++u) {
+        const int2 pu = __ldg(syz + u);
+        if (abs(pu.x - yh) > kWinY || abs(pu.y - zh) > kWinZ) continue;
+        for (int izd = dz0; izd <= dz1; ++izd) {
+          const int da = __ldg(cellStart + gd.cellBase + izd * gd.ny + dy0);
+          const int db = __ldg(cellStart + gd.cellBase + izd * gd.ny + dy1 + 1);
+          for (int d = da; d < db; ++d) {
+            const int2 pd = __ldg(syz + d);
+            if (abs(pd.x - yh) > kWinY || abs(pd.y - zh) > kWinZ) continue;
+            const int ey = y2 - pu.x - pd.x, ez = z2 - pu.y - pd.y;
+            const int D = kWeightY * ey * ey + kWeightZ * ez * ez;
+            if (D < bestD) {  // (u, d) visited in ascending order
+              bestD = D;
+              bu = u;
+              bd = d;
+            }
+          }
+        }
+      }
+    }
+  }
+}
+
+// One hit's best pair in the drift-ordered views of the adjacent rows,
+// candidates at positions [ua, ub) and [da, db).  The candidates of a side are
+// tested into a bit mask (no branch, loads independent), the one or two that
+// pass are fetched again: the lanes of a warp then differ only in short loops.
+// Sides of at most four candidates each (the common case) go through all 16
+// pairs in registers.  Equal metrics go to the smaller sorted up, then down
+// index.
+__device__ inline void nf_view(const ZView& V, const ZRow& gu, const ZRow& gd, int ua, int ub, int da, int db, int2 hh,
+                               int& bu, int& bd) {
+  const int2* pu = V.yz(gu);
+  const int2* pd = V.yz(gd);
+  const int* iu = V.idx(gu);
+  const int* id = V.idx(gd);
+  auto inside = [&](int2 c) {
+    return (unsigned)(hh.x - c.x + kWinY) <= 2u * kWinY && (unsigned)(hh.y - c.y + kWinZ) <= 2u * kWinZ;
+  };
+  auto metric = [&](int2 u, int2 d) {
+    const int ey = (hh.x - u.x) + (hh.x - d.x), ez = (hh.y - u.y) + (hh.y - d.y);
+    return kWeightY * ey * ey + kWeightZ * ez * ez;
+  };
+  int bestD = kMaxMetric + 1, pbu = -1, pbd = -1;
+  auto take = [&](int D, int u, int d) {
+    bool better = D < bestD;
+    if (D == bestD && pbu >= 0) {
+      const int a = __ldg(iu + u), b = __ldg(iu + pbu);
+      better = a < b || (a == b && __ldg(id + d) < __ldg(id + pbd));
+    }
+    if (better) {
+      bestD = D;
+      pbu = u;
+      pbd = d;
+    }
+  };
+  if (ub - ua <= 32 && db - da <= 32) {
+    auto mask = [&](const int2* p, int m) {
+      unsigned k = 0;
+#pragma unroll 4
+      for (int i = 0; i < m; ++i) k |= inside(__ldg(p + i)) ? 1u << i : 0u;
+      return k;
+    };
+    pu += ua;
+    pd += da;
+    const unsigned mu = mask(pu, ub - ua);
+    if (!mu) return;
+    const unsigned md = mask(pd, db - da);
+    if (!md) return;
+    if (__popc(mu) <= 4 && __popc(md) <= 4) {
+      // residuals of the four slots; an empty slot's y residual (700) puts
+      // every pair with it past the cut (700 - 240 = 460: 2077 * 460^2 > cut)
+      int uy[4], uz[4], dy[4], dz[4];
+      unsigned uPos = 0, dPos = 0, m = mu;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        uy[a] = 700;
+        uz[a] = 0;
+        if (m) {
+          const int i = __ffs(m) - 1;
+          m &= m - 1;
+          const int2 c = __ldg(pu + i);
+          uy[a] = hh.x - c.x;
+          uz[a] = hh.y - c.y;
+          uPos |= (unsigned)i << (8 * a);
+        }
+      }
+      m = md;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        dy[b] = 700;
+        dz[b] = 0;
+        if (m) {
+          const int i = __ffs(m) - 1;
+          m &= m - 1;
+          const int2 c = __ldg(pd + i);
+          dy[b] = hh.x - c.x;
+          dz[b] = hh.y - c.y;
+          dPos |= (unsigned)i << (8 * b);
+        }
+      }
+      unsigned D[16], best = ~0u;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const unsigned ey = (unsigned)(uy[k >> 2] + dy[k & 3]), ez = (unsigned)(uz[k >> 2] + dz[k & 3]);
+        D[k] = (unsigned)kWeightY * ey * ey + (unsigned)kWeightZ * ez * ez;
+        best = min(best, D[k]);
+      }
+      if (best > (unsigned)kMaxMetric) return;
+      unsigned eq = 0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) eq |= D[k] == best ? 1u << k : 0u;
+      bestD = (int)best;
+      do {  // one pair, or several of the same metric
+        const int k = __ffs(eq) - 1;
+        eq &= eq - 1;
+        const int u = (int)((uPos >> (8 * (k >> 2))) & 255u), d = (int)((dPos >> (8 * (k & 3))) & 255u);
+        if (pbu < 0) {
+          pbu = ua + u;
+          pbd = da + d;
+        } else {
+          take(bestD, ua + u, da + d);
+        }
+      } while (eq);
+    } else {
+      for (unsigned m = mu; m; m &= m - 1) {
+        const int u = __ffs(m) - 1;
+        const int2 cu = __ldg(pu + u);
+        for (unsigned n = md; n; n &= n - 1) {
+          const int d = __ffs(n) - 1;
+          take(metric(cu, __ldg(pd + d)), ua + u, da + d);
+        }
+      }
+    }
+  } else {
+    for (int u = ua; u < ub; ++u) {
+      const int2 cu = __ldg(pu + u);
+      if (!inside(cu)) continue;
+      for (int d = da; d < db; ++d) {
+        const int2 cd = __ldg(pd + d);
+        if (inside(cd)) take(metric(cu, cd), u, d);
+      }
+    }
+  }
+  if (pbu >= 0) {
+    bu = __ldg(iu + pbu);
+    bd = __ldg(id + pbd);
+  }
+}
+
+// K4: one thread per hit in the drift order of its row; blocks of kB hits
+// tile the rows (nfBlockStart, built for the same block size, maps a block to
+// its row, looked up once per block).  The hits of a warp are neighbours in
+// drift, so their candidates on an adjacent row are one run of 40-50 hits and
+// every lane's share of it is about equal: 8 candidates a side to test, against
+// 11 in the cells with the second cell row scanned by the few lanes that
+// reach it.  A hit next to a row flagged dense takes the cells.
+// Against the search in the cells: 1 ms frame (20.3 M clusters) 1.80 -> 1.01
+// ms, 32 orbits (59 M) 6.02 -> 3.80 ms; the views cost 0.16 and 0.56 ms.
+template <int kB>
+__global__ void __launch_bounds__(kB) k_neighbours_view(const RowGrid* __restrict__ grid,
+                                                        const int* __restrict__ nfBlockStart, int nRows,
+                                                        const int* __restrict__ cellStart,
+                                                        const int2* __restrict__ syz, const GeomConst* __restrict__ G,
+                                                        ZView zv, int* __restrict__ upRaw, int* __restrict__ dnRaw) {
+  if ((int)blockIdx.x >= nfBlockStart[nRows]) return;  // launched with an upper bound of blocks
+  __shared__ int s_row;
+  if (threadIdx.x == 0) s_row = upper_bound_i32(nfBlockStart, nRows + 1, blockIdx.x) - 1;
+  __syncthreads();
+  const int R = s_row;
+  const ZRow g = zv.rows[R];
+  const int q = (blockIdx.x - nfBlockStart[R]) * kB + threadIdx.x;
+  if (q >= g.count) return;
+  const int r = (R % kRowsPerTF) % kNRow;
+  if (r < 1 || r > kNRow - 2) {  // rows 0 and 151 get no links
+    upRaw[g.start + q] = -1;
+    dnRaw[g.start + q] = -1;
+    return;
+  }
+  const int2 hh = zv.yz(g)[q];
+  const int h = zv.idx(g)[q];
+  const ZRow gu = zv.rows[R + 1], gd = zv.rows[R - 1];
+  int bu = -1, bd = -1;
+  if ((gu.flags | gd.flags) & kZNFCells) {
+    const RowGrid cu = grid[R + 1], cd = grid[R - 1];
+    int uy0, uy1, uz0, uz1, dy0, dy1, dz0, dz1;
+    if (cell_range(cu, G->npads[r + 1], hh.x - kWinY, hh.x + kWinY, hh.y - kWinZ, hh.y + kWinZ, uy0, uy1, uz0, uz1) &&
+        cell_range(cd, G->npads[r - 1], hh.x - kWinY, hh.x + kWinY, hh.y - kWinZ, hh.y + kWinZ, dy0, dy1, dz0, dz1))
+      nf_cells(cu, cd, uy0, uy1, uz0, uz1, dy0, dy1, dz0, dz1, cellStart, syz, syz, 0, syz, 0, hh, bu, bd);
+  } else {
+    int ua, ub, da, db;
+    if (z_range(zv, gu, hh.y - kWinZ, hh.y + kWinZ, ua, ub) && z_range(zv, gd, hh.y - kWinZ, hh.y + kWinZ, da, db))
+      nf_view(zv, gu, gd, ua, ub, da, db, hh, bu, bd);
+  }
+  upRaw[h] = bu;
+  dnRaw[h] = bd;
+}
+
 // --- staging of the adjacent rows' candidate slabs (TMA bulk copy)
 constexpr int kSlab = 1024;            // staged hits per side (8 KB)
 constexpr int kSlabWaitLimit = 1 << 22;  // mbarrier polls before giving up on a copy
@@ -84,9 +322,8 @@ __device__ inline bool slab_wait(unsigned bar, int limit) {
   return false;
 }
 
-// K4: one thread per hit; blocks of kB hits tile the rows (nfBlockStart,
-// built for the same block size, maps a block to its row, looked up once per
-// block).  With kStage, the candidates come from shared memory: a block's
+// K4, staged form (o2tpc_config.nf_staged): one thread per hit in sorted
+// order, the candidate cells from shared memory: a block's
 // hits are consecutive in (cell, input) order, so they lie in the cell rows
 // between those of its first and last hit, and their candidates in the cell
 // rows of each adjacent pad row that this drift range (widened by the window)
@@ -95,17 +332,16 @@ __device__ inline bool slab_wait(unsigned bar, int limit) {
 // the range, completing on an mbarrier; the threads set up their windows
 // meanwhile and wait just before scanning.  A side whose range exceeds kSlab
 // hits (or a copy that does not complete within the wait limit, flagged in
-// err) reads global memory instead.  Without kStage every candidate is a
-// global (L1-cached) load.
-template <int kB, bool kStage>
-__global__ void __launch_bounds__(kB) k_neighbours(const RowGrid* __restrict__ grid,
+// err) reads global memory instead.
+template <int kB>
+__global__ void __launch_bounds__(kB) k_neighbours_staged(const RowGrid* __restrict__ grid,
                                                    const int* __restrict__ nfBlockStart, int nRows,
                                                    const int* __restrict__ cellStart, const int2* __restrict__ syz,
                                                    const GeomConst* __restrict__ G, int* __restrict__ upRaw,
                                                    int* __restrict__ dnRaw, unsigned* __restrict__ err,
                                                    unsigned inject) {
   if ((int)blockIdx.x >= nfBlockStart[nRows]) return;  // launched with an upper bound of blocks
-  __shared__ __align__(16) int2 s_slab[kStage ? 2 : 1][kStage ? kSlab : 1];
+  __shared__ __align__(16) int2 s_slab[2][kSlab];
   __shared__ __align__(8) unsigned long long s_bar;
   __shared__ int s_row, s_base[2], s_use[2];
   const unsigned bar = smem_addr(&s_bar);
@@ -114,7 +350,7 @@ __global__ void __launch_bounds__(kB) k_neighbours(const RowGrid* __restrict__ g
     s_row = R0;
     s_use[0] = s_use[1] = 0;
     const int r0 = (R0 % kRowsPerTF) % kNRow;
-    if (kStage && r0 >= 1 && r0 <= kNRow - 2) {
+    if (r0 >= 1 && r0 <= kNRow - 2) {
       const RowGrid g0 = grid[R0];
       const int hf = g0.start + (blockIdx.x - nfBlockStart[R0]) * kB;
       const int hl = min(hf + kB, g0.start + g0.count) - 1;
@@ -166,7 +402,7 @@ __global__ void __launch_bounds__(kB) k_neighbours(const RowGrid* __restrict__ g
     }
     return;
   }
-  const bool staged = kStage && (s_use[0] || s_use[1]);
+  const bool staged = s_use[0] || s_use[1];
   const int waitLimit = (inject & 1u) ? kSlabWaitInjected : kSlabWaitLimit;
   bool slabOk = true;
   int bu = -1, bd = -1;
@@ -184,66 +420,10 @@ __global__ void __launch_bounds__(kB) k_neighbours(const RowGrid* __restrict__ g
     }
     const int2* su = (staged && slabOk && s_use[0]) ? s_slab[0] : syz;
     const int bu0 = (staged && slabOk && s_use[0]) ? s_base[0] : 0;
-    const int2* sd = (staged && slabOk && s_use[1]) ? s_slab[kStage ? 1 : 0] : syz;
+    const int2* sd = (staged && slabOk && s_use[1]) ? s_slab[1] : syz;
     const int bd0 = (staged && slabOk && s_use[1]) ? s_base[1] : 0;
-    if (inWin) {
-      int ui[kNFCand] = {}, di[kNFCand] = {};
-      unsigned ur[kNFCand] = {}, dr[kNFCand] = {};
-      const int nu = nf_collect(gu, uy0, uy1, uz0, uz1, cellStart, su, bu0, hh, ui, ur);
-      const int nd = nu > 0 ? nf_collect(gd, dy0, dy1, dz0, dz1, cellStart, sd, bd0, hh, di, dr) : 0;
-      // bestD starts one above the cut, so "D < bestD" also applies the cut
-      int bestD = kMaxMetric + 1;
-      // pairs in ascending (u, d): a strict "<" keeps the first minimum,
-      // which is the lexicographic minimum of (D, u, d).  Slots [a0, kNFCand)
-      // of both sides: the last four when both sides fit there (the common
-      // case), else all of them.
-      auto pair_scan = [&](const int a0) {
-#pragma unroll
-        for (int a = a0; a < kNFCand; ++a)
-#pragma unroll
-          for (int b = a0; b < kNFCand; ++b) {
-            const unsigned sres = ur[a] + dr[b];
-            const int ey = (int)(sres >> 16) - 2048, ez = (int)(sres & 0xFFFFu) - 2048;
-            const int D = kWeightY * ey * ey + kWeightZ * ez * ez;
-            if (a >= kNFCand - nu && b >= kNFCand - nd && D < bestD) {
-              bestD = D;
-              bu = ui[a];
-              bd = di[b];
-            }
-          }
-      };
-      constexpr int kNFSmall = kNFCand < 4 ? kNFCand : 4;
-      if (nu <= kNFSmall && nd <= kNFSmall) {
-        pair_scan(kNFCand - kNFSmall);
-      } else if (nu <= kNFCand && nd <= kNFCand) {
-        pair_scan(0);
-      } else {
-        const int y2 = 2 * yh, z2 = 2 * zh;
-        for (int izu = uz0; izu <= uz1; ++izu) {
-          const int ua = __ldg(cellStart + gu.cellBase + izu * gu.ny + uy0);
-          const int ub = __ldg(cellStart + gu.cellBase + izu * gu.ny + uy1 + 1);
-          for (int u = ua; u < ub; ++u) {
-            const int2 pu = __ldg(syz + u);
-            if (abs(pu.x - yh) > kWinY || abs(pu.y - zh) > kWinZ) continue;
-            for (int izd = dz0; izd <= dz1; ++izd) {
-              const int da = __ldg(cellStart + gd.cellBase + izd * gd.ny + dy0);
-              const int db = __ldg(cellStart + gd.cellBase + izd * gd.ny + dy1 + 1);
-              for (int d = da; d < db; ++d) {
-                const int2 pd = __ldg(syz + d);
-                if (abs(pd.x - yh) > kWinY || abs(pd.y - zh) > kWinZ) continue;
-                const int ey = y2 - pu.x - pd.x, ez = z2 - pu.y - pd.y;
-                const int D = kWeightY * ey * ey + kWeightZ * ez * ez;
-                if (D < bestD) {  // (u, d) visited in ascending order
-                  bestD = D;
-                  bu = u;
-                  bd = d;
-                }
-              }
-            }
-          }
-        }
-      }
-    }
+    if (inWin)
+      nf_cells(gu, gd, uy0, uy1, uz0, uz1, dy0, dy1, dz0, dz1, cellStart, syz, su, bu0, sd, bd0, hh, bu, bd);
   }
   if (valid) {
     upRaw[h] = bu;
@@ -581,20 +761,21 @@ void launch_lower_bounds(const int* list, const int* nListDev, const int* keys, 
 }
 
 void launch_neighbours(int nfBlocks, int hitsPerBlock, bool stage, const RowGrid* grid, const int* nfBlockStart,
-                       int nRows, const int* cellStart, const int2* syz, const GeomConst* G, int* upRaw, int* dnRaw,
-                       unsigned* err, cudaStream_t st, unsigned inject) {
+                       int nRows, const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw,
+                       int* dnRaw, unsigned* err, cudaStream_t st, unsigned inject) {
   if (nfBlocks > 0) {
-#define O2TPC_NF(B, S) \
-  k_neighbours<B, S><<<nfBlocks, B, 0, st>>>(grid, nfBlockStart, nRows, cellStart, syz, G, upRaw, dnRaw, err, inject)
+#define O2TPC_NF(B)                                                                                                  \
+  if (stage)                                                                                                         \
+    k_neighbours_staged<B><<<nfBlocks, B, 0, st>>>(grid, nfBlockStart, nRows, cellStart, syz, G, upRaw, dnRaw, err,  \
+                                                   inject);                                                          \
+  else                                                                                                               \
+    k_neighbours_view<B><<<nfBlocks, B, 0, st>>>(grid, nfBlockStart, nRows, cellStart, syz, G, zv, upRaw, dnRaw)
     if (hitsPerBlock == 64) {
-      if (stage) O2TPC_NF(64, true);
-      else O2TPC_NF(64, false);
+      O2TPC_NF(64);
     } else if (hitsPerBlock == 256) {
-      if (stage) O2TPC_NF(256, true);
-      else O2TPC_NF(256, false);
+      O2TPC_NF(256);
     } else {
-      if (stage) O2TPC_NF(128, true);
-      else O2TPC_NF(128, false);
+      O2TPC_NF(128);
     }
 #undef O2TPC_NF
     ++g_launch_count;

@@ -346,8 +346,8 @@ void tune_cache_store(Ctx* c);
 // arrays as any other; the grid's block map is rebuilt for the chosen NF
 // shape before the real NeighboursFinder launch.
 void autotune(Ctx* c, int n, int nRows, const int* rowCnt, const int* rowMin, const int* rowMax, RowGrid* grid,
-              int* nfBlockStart, int* totals, const int4* bucket, int* cellStart, int2* syz, int* sorig,
-              int* gscratch, unsigned* err) {
+              int* nfBlockStart, int* totals, int4* bucket, int* cellStart, int2* syz, int* sorig, int* gscratch,
+              ZRow* zrow, unsigned* err) {
   cudaStream_t st = c->stream;
   const GeomConst* G = c->dGeom;
   static const int kSort[3] = {128, 256, 512};
@@ -366,12 +366,15 @@ void autotune(Ctx* c, int n, int nRows, const int* rowCnt, const int* rowMin, co
     launch_cell_sort(nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, kSort[i]);
     CK(cudaEventRecord(es[i][2], st));
   }
+  // the views take the place of the bucket records: after the last cell sort
+  launch_zorder(nRows, grid, rowMax, cellStart, syz, zrow, bucket, st);
+  const ZView zv{zrow, reinterpret_cast<const char*>(bucket)};
   for (int i = 0; i < 6; ++i) {
     const int hb = kNF[i % 3];
     launch_grid(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, hb, totals, st);
     const int blocks = n / hb + nRows + 1;
     CK(cudaEventRecord(en[i][0], st));
-    launch_neighbours(blocks, hb, i >= 3, grid, nfBlockStart, nRows, cellStart, syz, G, up, up + n, err, st);
+    launch_neighbours(blocks, hb, i >= 3, grid, nfBlockStart, nRows, cellStart, syz, G, zv, up, up + n, err, st);
     CK(cudaEventRecord(en[i][1], st));
   }
   CK(cudaEventSynchronize(en[5][1]));
@@ -681,12 +684,12 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   launch_row_scatter(dTF, dTiles, nTiles, tileSize, G, tileStats, grid, bucket, st);
   CKL();
   launch_cell_sort(nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, c->tune.sort_threads_per_row);
+  ZRow* zrow = dalloc<ZRow>(M, nRows);
   if ((c->cfg.flags & O2TPC_FLAG_AUTOTUNE) && !c->tune.tuned && n >= (1 << 20))
     autotune(c, n, nRows, rowCnt, rowMin, rowMax, grid, nfBlockStart, totals, bucket, cellStart, syz, sorig, gscratch,
-             dErr);
-  CKL();
-  ZRow* zrow = dalloc<ZRow>(M, nRows);
-  launch_zorder(nRows, grid, rowMax, cellStart, syz, zrow, bucket, st);
+             zrow, dErr);
+  else
+    launch_zorder(nRows, grid, rowMax, cellStart, syz, zrow, bucket, st);
   CKL();
   const ZView zv{zrow, reinterpret_cast<const char*>(bucket)};
 
@@ -700,8 +703,8 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   int* scratch = dalloc<int>(M, scan_scratch_ints((long long)n + 8) + (nRows + 8) * 2 / 4096 + 64);
   const int nfB = c->tune.nf_hits_per_block;
   const int nfBlocksMax = n / nfB + nRows + 1;
-  launch_neighbours(nfBlocksMax, nfB, c->tune.nf_staged != 0, grid, nfBlockStart, nRows, cellStart, syz, G, upRaw,
-                    dnRaw, dErr, st, c->cfg.debug_inject);
+  launch_neighbours(nfBlocksMax, nfB, c->tune.nf_staged != 0, grid, nfBlockStart, nRows, cellStart, syz, G, zv,
+                    upRaw, dnRaw, dErr, st, c->cfg.debug_inject);
   CKL();
   if (c->cfg.flags & O2TPC_FLAG_ROW_STEP2) {
     launch_neighbours_gap(n, &C->n, grid, nRows, cellStart, syz, G, upRaw, dnRaw, st);

@@ -181,7 +181,7 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   launch_zorder(k.nRows, A.grid, A.rowMax, A.cellStart, A.syz, A.zrow, A.bucket, st);
   const ZView zv{A.zrow, reinterpret_cast<const char*>(A.bucket)};
   // A5-A7
-  launch_neighbours(n / nfBlock + k.nRows + 1, nfBlock, nfStage, A.grid, A.nfBlockStart, k.nRows, A.cellStart, A.syz, G,
+  launch_neighbours(n / nfBlock + k.nRows + 1, nfBlock, nfStage, A.grid, A.nfBlockStart, k.nRows, A.cellStart, A.syz, G, zv,
                     A.upRaw, A.dnRaw, A.err, st);
   if (rowStep2) launch_neighbours_gap(n, &C->n, A.grid, k.nRows, A.cellStart, A.syz, G, A.upRaw, A.dnRaw, st);
   launch_clean(n, &C->n, A.upRaw, A.dnRaw, A.up, A.dn, A.flag, st);

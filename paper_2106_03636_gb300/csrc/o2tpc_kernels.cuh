@@ -37,8 +37,8 @@ void launch_zorder(int nRows, const RowGrid* grid, const int* rowMax, const int*
 // slab copies may read it); err collects kErrTimeout.  inject: the context's
 // debug_inject bits (bit 0: staged slabs armed but not copied, short waits).
 void launch_neighbours(int nfBlocks, int hitsPerBlock, bool stage, const RowGrid* grid, const int* nfBlockStart,
-                       int nRows, const int* cellStart, const int2* syz, const GeomConst* G, int* upRaw, int* dnRaw,
-                       unsigned* err, cudaStream_t st, unsigned inject = 0);
+                       int nRows, const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw,
+                       int* dnRaw, unsigned* err, cudaStream_t st, unsigned inject = 0);
 // Row step 2: links across one missing row for the hits that found no
 // adjacent-row pair (after launch_neighbours; n sizes the grid).
 void launch_neighbours_gap(int n, const int* nDev, const RowGrid* grid, int nRows, const int* cellStart,
