@@ -426,7 +426,7 @@ int o2tpc_get_tuning(o2tpc_ctx* ctx, o2tpc_tuning* out);
  * every device buffer, a fixed memory plan, code that must not synchronise
  * the device through cudaMalloc or grow its footprint after start-up): the
  * step's scratch memory is a set of file-scope static device arrays of fixed
- * size (about 6 MB, held by every GPU that loads the library until the
+ * size (about 8 MB, held by every GPU that loads the library until the
  * process exits), so this call allocates nothing, neither directly nor
  * through any allocating library routine.
  *
@@ -448,7 +448,7 @@ int o2tpc_get_tuning(o2tpc_ctx* ctx, o2tpc_tuning* out);
  * The static arrays' device addresses are looked up during the first call on
  * each device (with that device current), so make that first call before any
  * stream capture.  With CUDA's lazy module loading (the default) that first
- * call may also load the library's device code and reserve the ~6 MB of
+ * call may also load the library's device code and reserve the ~8 MB of
  * static storage at that moment: a caller with a fixed memory plan makes one
  * call with n = 0 at start-up (or runs with CUDA_MODULE_LOADING=EAGER).  The
  * looked-up addresses are kept for the life of the process and are not valid

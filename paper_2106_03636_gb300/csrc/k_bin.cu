@@ -8,6 +8,8 @@
 // per-(tile,row) prefix (no global atomics), then one CTA per row scatters
 // its bucket into cells and restores input order inside each cell, so the
 // result is the stable order whatever the atomic interleaving.
+#include <algorithm>
+
 #include "o2tpc_kernels.cuh"
 
 namespace o2tpc {
@@ -141,87 +143,99 @@ __global__ void __launch_bounds__(kRRRows * kRRChunks) k_row_reduce(const TFDesc
   }
 }
 
-// Block-wide exclusive scan of one int per thread (blockDim.x == 1024).
-__device__ inline int block_excl_scan(int v, int* total) {
-  __shared__ int ws[32];
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
+// Cells, NeighboursFinder blocks and grid of a row.
+__device__ inline RowGrid row_grid(int R, int nRows, const int* __restrict__ rowCnt, const int* __restrict__ rowMin,
+                                   const int* __restrict__ rowMax, const GeomConst* __restrict__ G) {
+  RowGrid g{};
+  if (R >= nRows) return g;  // no hits, no cells
+  const int n = rowCnt[R];
+  g.ny = max(1, (64 * G->npads[(R % kRowsPerTF) % kNRow] + kCellY - 1) / kCellY);
+  g.nz = 1;
+  g.cz = 1;
+  g.count = n;
+  if (n > 0) {
+    g.nz = min(max((n + kHitsPerCell * g.ny - 1) / (kHitsPerCell * g.ny), 1), kMaxNz);
+    // 1 .. 2^31 + 1 units over 1 .. 2^20 cells
+    const unsigned range = (unsigned)rowMax[R] - (unsigned)rowMin[R] + 1u;
+    g.cz = (int)((range + (unsigned)g.nz - 1u) / (unsigned)g.nz);
+    g.zmin = rowMin[R];
   }
-  if (lane == 31) ws[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int s = (lane < (int)(blockDim.x >> 5)) ? ws[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += y;
-    }
-    ws[lane] = s;
-  }
-  __syncthreads();
-  int incl = x + (w > 0 ? ws[w - 1] : 0);
-  if (total) *total = ws[(blockDim.x >> 5) - 1];
-  __syncthreads();
-  return incl - v;
+  return g;
 }
 
 // Grid of every row and the three row-level exclusive scans (hits, cells,
-// NeighboursFinder blocks).  One CTA of 1024 threads; each thread owns a
-// contiguous run of rows.  totals[0..2] = hits, cells, NF blocks.
-__global__ void __launch_bounds__(1024) k_grid(int nRows, const int* __restrict__ rowCnt, const int* __restrict__ rowMin,
-                                               const int* __restrict__ rowMax, const GeomConst* __restrict__ G,
-                                               RowGrid* __restrict__ grid, int* __restrict__ nfBlockStart,
-                                               int nfBlock, int* __restrict__ totals) {
-  int per = (nRows + blockDim.x - 1) / blockDim.x;
-  int b = threadIdx.x * per, e = min(nRows, b + per);
-  int sh = 0, sc = 0, sb = 0;
-  for (int R = b; R < e; ++R) {
-    int r = (R % kRowsPerTF) % kNRow;
-    int n = rowCnt[R];
-    int ny = max(1, (64 * G->npads[r] + kCellY - 1) / kCellY);
-    int nz = 1;
-    if (n > 0) nz = min(max((n + kHitsPerCell * ny - 1) / (kHitsPerCell * ny), 1), kMaxNz);
-    sh += n;
-    sc += ny * nz;
-    sb += (n + nfBlock - 1) / nfBlock;
+// NeighboursFinder blocks) in two launches of one thread per row: the sums of
+// every block of kGridRows rows, then each block adds up the sums before it
+// and scans its own rows.  totals[0..2] = hits, cells, NF blocks; sums:
+// 3 * grid_blocks(nRows) ints.  (One CTA over all rows, each thread walking
+// its run of rows twice, took 31 us for one Time Frame and 286 us for eight.)
+constexpr int kGridRows = 256;
+__global__ void __launch_bounds__(kGridRows) k_grid_sums(int nRows, const int* __restrict__ rowCnt,
+                                                         const int* __restrict__ rowMin,
+                                                         const int* __restrict__ rowMax,
+                                                         const GeomConst* __restrict__ G, int nfBlock,
+                                                         int* __restrict__ sums) {
+  __shared__ int ws[3][kGridRows / 32];
+  const RowGrid g = row_grid(blockIdx.x * kGridRows + threadIdx.x, nRows, rowCnt, rowMin, rowMax, G);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int v[3] = {g.count, g.ny * g.nz, (g.count + nfBlock - 1) / nfBlock};
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int x = __reduce_add_sync(0xffffffffu, v[q]);
+    if (lane == 0) ws[q][w] = x;
   }
-  int th, tc, tb;
-  int oh = block_excl_scan(sh, &th);
-  int oc = block_excl_scan(sc, &tc);
-  int ob = block_excl_scan(sb, &tb);
-  for (int R = b; R < e; ++R) {
-    int r = (R % kRowsPerTF) % kNRow;
-    int n = rowCnt[R];
-    RowGrid g;
-    g.ny = max(1, (64 * G->npads[r] + kCellY - 1) / kCellY);
-    g.nz = 1;
-    g.cz = 1;
-    g.zmin = 0;
-    if (n > 0) {
-      g.nz = min(max((n + kHitsPerCell * g.ny - 1) / (kHitsPerCell * g.ny), 1), kMaxNz);
-      long long range = (long long)rowMax[R] - (long long)rowMin[R] + 1;
-      g.cz = (int)((range + g.nz - 1) / g.nz);
-      g.zmin = rowMin[R];
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    int s = 0;
+    for (int k = 0; k < kGridRows / 32; ++k) s += ws[threadIdx.x][k];
+    sums[threadIdx.x * gridDim.x + blockIdx.x] = s;
+  }
+}
+
+__global__ void __launch_bounds__(kGridRows) k_grid(int nRows, const int* __restrict__ rowCnt, const int* __restrict__ rowMin,
+                                                    const int* __restrict__ rowMax, const GeomConst* __restrict__ G,
+                                                    RowGrid* __restrict__ grid, int* __restrict__ nfBlockStart,
+                                                    int nfBlock, const int* __restrict__ sums,
+                                                    int* __restrict__ totals) {
+  __shared__ int ws[3][kGridRows / 32], base[3][kGridRows / 32];
+  const int R = blockIdx.x * kGridRows + threadIdx.x;
+  RowGrid g = row_grid(R, nRows, rowCnt, rowMin, rowMax, G);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int v[3] = {g.count, g.ny * g.nz, (g.count + nfBlock - 1) / nfBlock};
+  int x[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    int b = 0;  // of the blocks before
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += kGridRows) b += sums[q * gridDim.x + k];
+    b = __reduce_add_sync(0xffffffffu, b);
+    x[q] = v[q];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x[q], o);
+      if (lane >= o) x[q] += y;
     }
-    g.start = oh;
-    g.count = n;
-    g.cellBase = oc;
-    g.pad = 0;
-    grid[R] = g;
-    nfBlockStart[R] = ob;
-    oh += n;
-    oc += g.ny * g.nz;
-    ob += (n + nfBlock - 1) / nfBlock;
+    if (lane == 31) {
+      ws[q][w] = x[q];
+      base[q][w] = b;
+    }
   }
-  if (threadIdx.x == 0) {
-    totals[0] = th;
-    totals[1] = tc;
-    totals[2] = tb;
-    nfBlockStart[nRows] = tb;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    x[q] -= v[q];
+    for (int k = 0; k < kGridRows / 32; ++k) x[q] += base[q][k] + (k < w ? ws[q][k] : 0);
+  }
+  if (R < nRows) {
+    g.start = x[0];
+    g.cellBase = x[1];
+    grid[R] = g;
+    nfBlockStart[R] = x[2];
+    if (R == nRows - 1) {
+      totals[0] = x[0] + v[0];
+      totals[1] = x[1] + v[1];
+      totals[2] = x[2] + v[2];
+      nfBlockStart[nRows] = x[2] + v[2];
+    }
   }
 }
 
@@ -514,8 +528,30 @@ void launch_row_reduce(const TFDesc* tfs, int nTF, int* tileStats, int* rowCnt, 
 
 void launch_grid(int nRows, const int* rowCnt, const int* rowMin, const int* rowMax, const GeomConst* G,
                  RowGrid* grid, int* nfBlockStart, int nfBlock, int* totals, cudaStream_t st) {
-  k_grid<<<1, 1024, 0, st>>>(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, nfBlock, totals);
-  ++g_launch_count;
+  if (nRows <= 0) return;
+  int* sums = totals + 4;
+  const int nb = grid_blocks(nRows);
+  k_grid_sums<<<nb, kGridRows, 0, st>>>(nRows, rowCnt, rowMin, rowMax, G, nfBlock, sums);
+  k_grid<<<nb, kGridRows, 0, st>>>(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, nfBlock, sums, totals);
+  g_launch_count += 2;
+}
+
+int grid_blocks(int nRows) { return (nRows + kGridRows - 1) / kGridRows; }
+
+// Tiles: their number bounds the parallelism of the ingest and of the scatter
+// (a CTA takes tiles in turn), each costs 64 KB of row statistics written and
+// read.  Four tiles per SM, of 8192 to 65536 clusters: with 65536 throughout,
+// 1.3 M clusters gave 20 tiles to 152 SMs (ingest 84, scatter 131 us), and the
+// 310 tiles of 20 M clusters left the scatter's last round nearly empty.
+int ingest_tile(long long n) {
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 148;
+  }();
+  const long long t = (n + 4ll * sms - 1) / (4ll * sms);
+  return (int)std::min<long long>(std::max<long long>((t + 255) / 256 * 256, kTileMin), kTileMax);
 }
 
 // CTAs per SM of the persistent row scatter

@@ -58,7 +58,6 @@ void o2tpc::fill_geom(GeomConst& g, double bz, double vd) {
 
 namespace {
 
-constexpr int kTileMin = 65536;           // clusters per ingest tile, at least
 constexpr int kTilesPerTFMax = 4096;
 constexpr uint64_t kMaxBatchHits = 2000000000ull;
 // With the compressed TF: the blob offsets are 32-bit, and a coded cluster
@@ -612,20 +611,15 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
       input_upload(t, p, st);
       input_layout(t, p, d);
     }
-    int tileSize = std::max(kTileMin, (int)((t.n + kTilesPerTFMax - 1) / kTilesPerTFMax));
-    d.tileBase = (int)tiles.size();
-    d.nTiles = (int)((t.n + tileSize - 1) / tileSize);
-    for (int k = 0; k < d.nTiles; ++k) tiles.push_back(make_int2(i, k * tileSize));
     d.nColl = (int)t.n_coll;
     d.collBase = nColl;
     nColl += (int)t.n_coll;
     tfd[i] = d;
     N += (long long)t.n;
   }
-  // one tile size for the launch: the largest any TF asked for
-  int tileSize = kTileMin;
+  // one tile size for the launch
+  int tileSize = ingest_tile(N);
   for (int i = 0; i < B; ++i) tileSize = std::max(tileSize, (int)((jobs[i]->tf.n + kTilesPerTFMax - 1) / kTilesPerTFMax));
-  tiles.clear();
   for (int i = 0; i < B; ++i) {
     tfd[i].tileBase = (int)tiles.size();
     tfd[i].nTiles = (int)((jobs[i]->tf.n + tileSize - 1) / tileSize);
@@ -667,7 +661,7 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   int* rowMax = dalloc<int>(M, nRows);
   RowGrid* grid = dalloc<RowGrid>(M, nRows + 1);
   int* nfBlockStart = dalloc<int>(M, nRows + 1);
-  int* totals = dalloc<int>(M, 4);
+  int* totals = dalloc<int>(M, 4 + 3 * grid_blocks(nRows));
   launch_ingest_stats(dTF, dTiles, nTiles, tileSize, G, tileStats, dErr, st);
   CKL();
   launch_row_reduce(dTF, B, tileStats, rowCnt, rowMin, rowMax, st);

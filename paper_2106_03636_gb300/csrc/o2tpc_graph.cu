@@ -24,7 +24,7 @@ GraphCaps graph_caps(long long maxClusters, int maxTFs, bool tight) {
   GraphCaps k{};
   k.nCap = (int)std::max<long long>(maxClusters, 1);
   k.BCap = std::max(maxTFs, 1);
-  k.tileSize = kGraphTile;
+  k.tileSize = ingest_tile(k.nCap);
   k.nTilesCap = k.nCap / k.tileSize + k.BCap + 1;
   k.nRows = k.BCap * kRowsPerTF;
   k.cellsCap = (long long)k.nCap / kHitsPerCell + 46ll * k.nRows + 1;
@@ -63,7 +63,7 @@ size_t graph_carve(GraphArena& A, char* base) {
   take(A.rowMax, k.nRows);
   take(A.grid, k.nRows + 1);
   take(A.nfBlockStart, k.nRows + 1);
-  take(A.totals, 4);
+  take(A.totals, 4 + 3 * grid_blocks(k.nRows));
   take(A.cellStart, k.cellsCap + 1);
   take(A.gscratch, k.cellsCap);
   take(A.bucket, n);

@@ -5,8 +5,6 @@
 
 namespace o2tpc {
 
-constexpr int kGraphTile = 65536;  // clusters per ingest tile on the captured path
-
 // Capacities of a captured-path arena (from the largest batch it serves).
 struct GraphCaps {
   int nCap, BCap, tileSize, nTilesCap, nRows;

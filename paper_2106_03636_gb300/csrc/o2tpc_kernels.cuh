@@ -19,6 +19,11 @@ void launch_ingest_stats(const TFDesc* tfs, const int2* tiles, int nTiles, int t
                          int* tileStats, unsigned* err, cudaStream_t st);
 void launch_row_reduce(const TFDesc* tfs, int nTF, int* tileStats, int* rowCnt, int* rowMin, int* rowMax,
                        cudaStream_t st);
+// totals: 4 ints, then 3 * grid_blocks(nRows) of scratch.
+int grid_blocks(int nRows);
+// Clusters per ingest tile of a batch of n clusters.
+constexpr int kTileMin = 8192, kTileMax = 65536;
+int ingest_tile(long long n);
 void launch_grid(int nRows, const int* rowCnt, const int* rowMin, const int* rowMax, const GeomConst* G,
                  RowGrid* grid, int* nfBlockStart, int nfBlock, int* totals, cudaStream_t st);
 void launch_row_scatter(const TFDesc* tfs, const int2* tiles, int nTiles, int tileSize, const GeomConst* G,

@@ -13,7 +13,7 @@
 // device arrays of fixed size, so the call allocates nothing.
 //
 // The arrays are static __device__ storage: every GPU that loads the library
-// holds them (about 6 MB) until the process exits.  Their device addresses
+// holds them (about 8 MB) until the process exits.  Their device addresses
 // are looked up once per device with cudaGetSymbolAddress, during the first
 // call on that device; that first call should therefore come before any
 // stream capture.  Under lazy module loading that first call can also load
@@ -32,7 +32,7 @@
 namespace o2tpc {
 namespace {
 
-constexpr int kStaticTile = 65536;
+constexpr int kStaticTile = kTileMin;
 constexpr int kStaticTiles = (O2TPC_STATIC_MAX_CLUSTERS + kStaticTile - 1) / kStaticTile;
 constexpr long long kStaticCells = O2TPC_STATIC_MAX_CLUSTERS / kHitsPerCell + 46ll * kRowsPerTF + 1;
 
@@ -44,7 +44,7 @@ static __device__ __align__(256) int s_rowCnt[kRowsPerTF];
 static __device__ __align__(256) int s_rowMin[kRowsPerTF];
 static __device__ __align__(256) int s_rowMax[kRowsPerTF];
 static __device__ __align__(256) int s_nfBlockStart[kRowsPerTF + 1];
-static __device__ __align__(256) int s_totals[4];
+static __device__ __align__(256) int s_totals[4 + 3 * ((kRowsPerTF + 255) / 256)];
 static __device__ __align__(256) unsigned s_err[4];
 static __device__ __align__(256) int4 s_bucket[O2TPC_STATIC_MAX_CLUSTERS];
 static __device__ __align__(256) int s_cellScratch[kStaticCells];
