@@ -247,6 +247,24 @@ __device__ inline void nf_view(const ZView& V, const ZRow& gu, const ZRow& gd, i
   }
 }
 
+// First index of a[0, n) with a[i] > v, searched by the whole warp: 32 probes
+// a step, 3-4 dependent loads where a binary search takes 13-18 (all lanes
+// must call it; every lane gets the result).
+__device__ inline int warp_upper_bound(const int* __restrict__ a, int n, int v) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, hi = n;  // answer in [lo, hi]
+  while (hi > lo) {
+    const int step = (hi - lo + 31) / 32;
+    const int i = lo + lane * step;  // ascending probes
+    const unsigned m = __ballot_sync(0xffffffffu, i < hi && a[i] <= v);
+    const int k = __popc(m);  // probes at or below v
+    if (k == 0) return lo;
+    lo += (k - 1) * step + 1;
+    hi = min(hi, lo + step - 1);
+  }
+  return lo;
+}
+
 // K4: one thread per hit in the drift order of its row; blocks of kB hits
 // tile the rows (nfBlockStart, built for the same block size, maps a block to
 // its row, looked up once per block).  The hits of a warp are neighbours in
@@ -254,8 +272,8 @@ __device__ inline void nf_view(const ZView& V, const ZRow& gu, const ZRow& gd, i
 // every lane's share of it is about equal: 8 candidates a side to test, against
 // 11 in the cells with the second cell row scanned by the few lanes that
 // reach it.  A hit next to a row flagged dense takes the cells.
-// Against the search in the cells: 1 ms frame (20.3 M clusters) 1.80 -> 1.01
-// ms, 32 orbits (59 M) 6.02 -> 3.80 ms; the views cost 0.16 and 0.56 ms.
+// Against the search in the cells: 1 ms frame (20.3 M clusters) 1.80 -> 0.94
+// ms, 32 orbits (59 M) 6.02 -> 3.63 ms; the views cost 0.16 and 0.56 ms.
 template <int kB>
 __global__ void __launch_bounds__(kB) k_neighbours_view(const RowGrid* __restrict__ grid,
                                                         const int* __restrict__ nfBlockStart, int nRows,
@@ -263,10 +281,7 @@ __global__ void __launch_bounds__(kB) k_neighbours_view(const RowGrid* __restric
                                                         const int2* __restrict__ syz, const GeomConst* __restrict__ G,
                                                         ZView zv, int* __restrict__ upRaw, int* __restrict__ dnRaw) {
   if ((int)blockIdx.x >= nfBlockStart[nRows]) return;  // launched with an upper bound of blocks
-  __shared__ int s_row;
-  if (threadIdx.x == 0) s_row = upper_bound_i32(nfBlockStart, nRows + 1, blockIdx.x) - 1;
-  __syncthreads();
-  const int R = s_row;
+  const int R = warp_upper_bound(nfBlockStart, nRows + 1, blockIdx.x) - 1;
   const ZRow g = zv.rows[R];
   const int q = (blockIdx.x - nfBlockStart[R]) * kB + threadIdx.x;
   if (q >= g.count) return;
