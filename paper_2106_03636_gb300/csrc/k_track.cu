@@ -280,9 +280,10 @@ __device__ inline unsigned long long cand_key(int h, int2 p, const SearchPar& P,
   return ((unsigned long long)__float_as_uint(chi) << 32) | (unsigned)h;
 }
 
-// Best hit of a search: its sorted index (-1: none) and coordinates.
+// Best hit of a search: its index in the list `idx` of sorted indices (null:
+// it is the sorted index itself; -1: none) and its coordinates.
 struct BestHit {
-  int hit;
+  int pos;
   int2 p;
 };
 
@@ -302,7 +303,7 @@ __device__ inline BestHit cell_search(const RowGrid& g, int iy0, int iy1, int iz
       const unsigned long long key = cand_key(h, p, P, zunit);
       if (key < best) {
         best = key;
-        B.hit = h;
+        B.pos = h;
         B.p = p;
       }
     }
@@ -312,13 +313,12 @@ __device__ inline BestHit cell_search(const RowGrid& g, int iy0, int iy1, int iz
 
 // Per-lane search through positions [a, b) of a row's drift-ordered view:
 // four candidates loaded at once (a window holds 3-4 on average), so a row
-// step waits for one load and not for one per candidate.  Equal chi2 goes to
-// the smaller sorted index.
-__device__ inline BestHit z_search(const ZView& V, const ZRow& g, int a, int b, const SearchPar& P, float zunit) {
-  const int2* yz = V.yz(g);
-  const int* idx = V.idx(g);
+// step waits for one load and not for one per candidate.  Equal chi2 (rare)
+// goes to the smaller sorted index.
+__device__ inline BestHit z_search(const int2* __restrict__ yz, const int* __restrict__ idx, int a, int b,
+                                   const SearchPar& P, float zunit) {
   unsigned best = ~0u;
-  int pos = -1;
+  bool tie = false;
   BestHit B{-1, make_int2(0, 0)};
   for (int h = a; h < b; h += 4) {
     int2 q[4];
@@ -326,20 +326,29 @@ __device__ inline BestHit z_search(const ZView& V, const ZRow& g, int a, int b, 
     for (int u = 0; u < 4; ++u) q[u] = __ldg(yz + min(h + u, b - 1));
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const unsigned long long key = cand_key(0, q[u], P, zunit);
-      const unsigned c = (unsigned)(key >> 32);
-      if (key != kNoHit && h + u < b) {
-        bool take = c < best;
-        if (c == best) take = __ldg(idx + h + u) < __ldg(idx + pos);
-        if (take) {
-          best = c;
-          pos = h + u;
-          B.p = q[u];
-        }
+      // as cand_key, without branches
+      const float dy = __fsub_rn(__fmul_rn((float)(q[u].x - P.yref), 0.00625f), P.y);
+      const float dz = __fsub_rn(__fmul_rn((float)(q[u].y - P.zref), zunit), P.z);
+      const float chi = __fadd_rn(__fmul_rn(__fmul_rn(dy, dy), P.isy2), __fmul_rn(__fmul_rn(dz, dz), P.isz2));
+      const bool ok = (h + u < b) & (fabsf(dy) <= P.wy) & (fabsf(dz) <= P.wz) & (chi <= kChi2Follow);
+      const unsigned c = ok ? __float_as_uint(chi) : ~0u;
+      tie |= ok & (c == best);
+      const bool take = c < best;
+      best = take ? c : best;
+      B.pos = take ? h + u : B.pos;
+      B.p.x = take ? q[u].x : B.p.x;
+      B.p.y = take ? q[u].y : B.p.y;
+    }
+  }
+  if (tie) {
+    for (int h = a; h < b; ++h) {
+      const int2 q = __ldg(yz + h);
+      if ((unsigned)(cand_key(0, q, P, zunit) >> 32) == best && __ldg(idx + h) < __ldg(idx + B.pos)) {
+        B.pos = h;
+        B.p = q;
       }
     }
   }
-  if (pos >= 0) B.hit = __ldg(idx + pos);
   return B;
 }
 
@@ -543,10 +552,13 @@ __global__ void __launch_bounds__(128, 7) k_tl_follow_coop(const int* __restrict
 // direction parameters and the row of the last accepted state (with kKeep the
 // whole state, for inspection), so nothing is copied per accepted hit.
 // Measured against the search in the cells with the state copied per hit:
-// 1 ms frame (20.3 M clusters) 2.26 + 1.73 -> 1.66 + 1.40 ms, 32 orbits (59 M)
-// 6.87 + 5.19 -> 4.98 + 4.12 ms, 3 collisions (1.3 M, one tracklet a lane)
-// 0.58 + 0.55 -> 0.43 + 0.48 ms.
-// Blocks of 128 per SM the kernel is compiled for:
+// 1 ms frame (20.3 M clusters) 2.26 + 1.73 -> 1.59 + 1.31 ms, 32 orbits (59 M)
+// 6.87 + 5.19 -> 4.73 + 3.97 ms, 3 collisions (1.3 M, one tracklet a lane)
+// 0.58 + 0.55 -> 0.37 + 0.45 ms.
+// The list index of the hit is loaded off the step's chain (beside the
+// update).  Loading the next row's bin starts ahead (prefetch to L1 or L2) cost
+// 6 %.  Blocks of 128 per SM the kernel is compiled for: 7 (72 registers)
+// measured 1.58 + 1.32 ms, 8 1.73 + 1.42, 6 1.59 + 1.36.
 #ifndef O2TPC_FOLLOW_MIN_BLOCKS
 #define O2TPC_FOLLOW_MIN_BLOCKS 7
 #endif
@@ -631,6 +643,7 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
     }
     // one row step of every busy lane: transport, then the window
     BestHit best{-1, make_int2(0, 0)};
+    const int* idx = nullptr;
     if (have) {
       if ((kDir > 0) ? (r >= kNRow) : (r < 0)) {
         finish();
@@ -650,17 +663,21 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
               best = cell_search(gc, iy0, iy1, iz0, iz1, cellStart, syz, P, zunit);
           } else {
             int a, b;
-            if (z_range(zv, g, zlo, zhi, a, b)) best = z_search(zv, g, a, b, P, zunit);
+            if (z_range(zv, g, zlo, zhi, a, b)) {
+              idx = zv.idx(g);
+              best = z_search(zv.yz(g), idx, a, b, P, zunit);
+            }
           }
         }
       }
     }
     if (have) {
-      if (best.hit >= 0) {
+      if (best.pos >= 0) {
+        const int hit = idx ? __ldg(idx + best.pos) : best.pos;  // in flight during the update
         recentre_y(st.p[0], yref, best.p.x);
         kf_update<float>(st, hit_y(best.p.x, yref), hit_z(best.p.y, zref, zunit), nullptr, angErr);
-        tb.hits[(size_t)k * kMaxTlHits + n] = best.hit;
         tb.rows[(size_t)k * kMaxTlHits + n] = (uint8_t)r;
+        tb.hits[(size_t)k * kMaxTlHits + n] = hit;
         ++n;
         save_last();
         misses = 0;
