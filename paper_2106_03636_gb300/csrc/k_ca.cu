@@ -654,62 +654,47 @@ void scan_exclusive(const int* in, int* out, int n, const int* nDev, int* scratc
   ++g_launch_count;
 }
 
-// ---- processing order by length (longest first)
-__device__ inline int len_bin(const int* __restrict__ off, int i) {
-  return kLenBins - 1 - min(off[i + 1] - off[i], kLenBins - 1);
-}
-
-__global__ void __launch_bounds__(256) k_len_hist(const int* __restrict__ nDev, const int* __restrict__ off,
-                                                  int* __restrict__ hist) {
-  __shared__ int sh[kLenBins];
-  for (int b = threadIdx.x; b < kLenBins; b += blockDim.x) sh[b] = 0;
+// ---- processing order by length
+// A block orders its kOrderChunk consecutive items longest first (a counting
+// sort in shared memory).
+constexpr int kOrderChunk = 1024, kOrderBins = 256;
+__global__ void __launch_bounds__(kOrderChunk) k_length_order(const int* __restrict__ nDev, const int* __restrict__ a,
+                                                              int diff, int* __restrict__ perm) {
+  __shared__ int hist[kOrderBins];
+  const int n = *nDev, base = blockIdx.x * kOrderChunk, i = base + threadIdx.x;
+  if (base >= n) return;
+  for (int b = threadIdx.x; b < kOrderBins; b += kOrderChunk) hist[b] = 0;
   __syncthreads();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < *nDev) atomicAdd(&sh[len_bin(off, i)], 1);
-  __syncthreads();
-  for (int b = threadIdx.x; b < kLenBins; b += blockDim.x)
-    if (sh[b]) atomicAdd(&hist[b], sh[b]);
-}
-
-// hist[0, kLenBins) -> exclusive offsets (one CTA of kLenBins threads)
-__global__ void __launch_bounds__(kLenBins) k_len_scan(int* __restrict__ hist) {
-  __shared__ int sh[kLenBins];
-  const int v = hist[threadIdx.x];
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int d = 1; d < kLenBins; d <<= 1) {
-    const int t = threadIdx.x >= d ? sh[threadIdx.x - d] : 0;
-    __syncthreads();
-    sh[threadIdx.x] += t;
-    __syncthreads();
+  int bin = -1, rank = 0;
+  if (i < n) {
+    const int len = diff ? a[i + 1] - a[i] : a[i];
+    bin = kOrderBins - 1 - min(max(len, 0), kOrderBins - 1);
+    rank = atomicAdd(&hist[bin], 1);
   }
-  hist[threadIdx.x] = sh[threadIdx.x] - v;
+  __syncthreads();
+  if (threadIdx.x < 32) {  // exclusive scan of the bins
+    constexpr int per = kOrderBins / 32;
+    int v[per], sum = 0;
+#pragma unroll
+    for (int q = 0; q < per; ++q) {
+      v[q] = hist[threadIdx.x * per + q];
+      sum += v[q];
+    }
+    int x = warp_incl(sum) - sum;
+#pragma unroll
+    for (int q = 0; q < per; ++q) {
+      hist[threadIdx.x * per + q] = x;
+      x += v[q];
+    }
+  }
+  __syncthreads();
+  if (bin >= 0) perm[base + hist[bin] + rank] = i;
 }
 
-// Each block ranks its items per bin in shared memory, then reserves its
-// range in each bin with one global atomic per (block, bin).
-__global__ void __launch_bounds__(1024) k_len_place(const int* __restrict__ nDev, const int* __restrict__ off,
-                                                    int* __restrict__ hist, int* __restrict__ perm) {
-  __shared__ int sh[kLenBins];
-  for (int b = threadIdx.x; b < kLenBins; b += blockDim.x) sh[b] = 0;
-  __syncthreads();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int bin = (i < *nDev) ? len_bin(off, i) : -1;
-  const int rank = (bin >= 0) ? atomicAdd(&sh[bin], 1) : 0;
-  __syncthreads();
-  for (int b = threadIdx.x; b < kLenBins; b += blockDim.x)
-    if (sh[b]) sh[b] = atomicAdd(&hist[b], sh[b]);
-  __syncthreads();
-  if (bin >= 0) perm[sh[bin] + rank] = i;
-}
-
-void launch_len_order(int n, const int* nDev, const int* off, int* hist, int* perm, cudaStream_t st) {
+void launch_length_order(int n, const int* nDev, const int* a, bool diff, int* perm, cudaStream_t st) {
   if (n <= 0) return;
-  cudaMemsetAsync(hist, 0, sizeof(int) * kLenBins, st);
-  k_len_hist<<<(n + 255) / 256, 256, 0, st>>>(nDev, off, hist);
-  k_len_scan<<<1, kLenBins, 0, st>>>(hist);
-  k_len_place<<<(n + 1023) / 1024, 1024, 0, st>>>(nDev, off, hist, perm);
-  g_launch_count += 3;
+  k_length_order<<<(n + kOrderChunk - 1) / kOrderChunk, kOrderChunk, 0, st>>>(nDev, a, diff ? 1 : 0, perm);
+  ++g_launch_count;
 }
 
 // *dst = min(arr[*idx], cap) (a count read off the end of a scan), flagging

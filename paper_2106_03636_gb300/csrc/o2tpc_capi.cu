@@ -731,8 +731,9 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   tb.zref = dalloc<int>(M, nTl);
   tb.yref = dalloc<int>(M, nTl);
   tb.rbase = dalloc<int>(M, nTl);
-  int* workCounter = dalloc<int>(M, 4);
-  launch_tracklets(nTl, &C->nTl, workCounter, starts, up, grid, nRows, cellStart, syz, G, zv, tb, st, c->evTl,
+  int* workCounter = dalloc<int>(M, kWorkCounters);
+  int* tlPerm = dalloc<int>(M, nTl);
+  launch_tracklets(nTl, &C->nTl, workCounter, starts, up, grid, nRows, cellStart, syz, G, zv, tb, tlPerm, st, c->evTl,
                    (c->cfg.flags & O2TPC_FLAG_COOP_SEARCH) != 0, (c->cfg.flags & O2TPC_FLAG_KEEP_STAGES) != 0);
   CKL();
 
@@ -781,10 +782,8 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   launch_st_gather(nStHits, &C->nStHits, sb, syz, sorig, st);
   CKL();
   CK(cudaEventRecord(c->evs[6], st));
-  int* lenHist = dalloc<int>(M, kLenBins);
-  int* stOrder = dalloc<int>(M, nSt);
-  launch_len_order(nSt, &C->nSt, sb.off, lenHist, stOrder, st);
-  launch_sector_fit(nSt, &C->nSt, tb, syz, G, sb, stOrder, st);
+  int* stPerm = dalloc<int>(M, nSt);
+  launch_sector_fit(nSt, &C->nSt, workCounter + 4, stPerm, tb, G, sb, st);
   CKL();
   int* stTfBegin = dalloc<int>(M, B + 1);
   int* tfKeys = dalloc<int>(M, B + 1);
@@ -874,8 +873,8 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   CKL();
   scan_exclusive(trkNcl, ob.off, nHeads, &C->nHeads, scratch, st);
   CKL();
-  launch_final_refit(nHeads, &C->nHeads, heads, sb, mb, syz, sorig, dTF, G,
-                     (c->cfg.flags & O2TPC_FLAG_FORCE_FP64) ? 1 : 0, ob, st);
+  launch_final_refit(nHeads, &C->nHeads, nSt, heads, sb, mb, syz, dTF, G,
+                     (c->cfg.flags & O2TPC_FLAG_FORCE_FP64) ? 1 : 0, workCounter + 5, stPerm, ob, st);
   CKL();
   int* trkTfBegin = dalloc<int>(M, B + 1);
   launch_lower_bounds(heads, &C->nHeads, stTfBegin, B + 1, trkTfBegin, st);

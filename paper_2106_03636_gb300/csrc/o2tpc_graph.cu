@@ -88,7 +88,8 @@ size_t graph_carve(GraphArena& A, char* base) {
   take(A.tb.zref, k.tlCap);
   take(A.tb.yref, k.tlCap);
   take(A.tb.rbase, k.tlCap);
-  take(A.workCounter, 4);
+  take(A.workCounter, kWorkCounters);
+  take(A.perm, std::max(k.tlCap, k.stCap));
   take(A.w, n);
   take(A.secBegin, k.BCap * kNSec + 1);
   take(A.wide, 1);
@@ -151,8 +152,6 @@ size_t graph_carve(GraphArena& A, char* base) {
     take(o->coll, k.headCap);
   }
   take(A.trkTfBegin, k.BCap + 1);
-  take(A.lenHist, kLenBins);
-  take(A.stOrder, k.stCap);
   take(A.coll, k.collCap);
   take(A.memNext, k.headCap);
   take(A.memPrev, k.headCap);
@@ -190,7 +189,7 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   launch_tf_ranges(k.BCap, A.grid, A.starts, &C->nTl, A.tlTfBegin, st);
   // A8
   launch_tracklets(k.tlCap, &C->nTl, A.workCounter, A.starts, A.up, A.grid, k.nRows, A.cellStart, A.syz, G, zv,
-                   A.tb, st, nullptr, coopSearch);
+                   A.tb, A.perm, st, nullptr, coopSearch);
   // A9
   cudaMemsetAsync(A.w, 0, sizeof(unsigned long long) * (size_t)n, st);
   launch_ownership(k.tlCap, &C->nTl, k.BCap * kNSec, A.grid, A.starts, A.tb, A.w, A.secBegin, A.wide, st);
@@ -202,8 +201,7 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   launch_count_at(A.segPos, &C->nTl, &C->nSt, k.stCap, &C->overflow, st, A.segHitPos, &C->nStHits, k.stHitsCap,
                   A.sb.off);
   launch_st_gather(k.stHitsCap, &C->nStHits, A.sb, A.syz, A.sorig, st);
-  launch_len_order(k.stCap, &C->nSt, A.sb.off, A.lenHist, A.stOrder, st);
-  launch_sector_fit(k.stCap, &C->nSt, A.tb, A.syz, G, A.sb, A.stOrder, st);
+  launch_sector_fit(k.stCap, &C->nSt, A.workCounter + 4, A.perm, A.tb, G, A.sb, st);
   launch_iota(A.tfKeys, k.BCap + 1, st);
   launch_lower_bounds(A.sb.tf, &C->nSt, A.tfKeys, k.BCap + 1, A.stTfBegin, st);
   // A10
@@ -218,7 +216,8 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   cudaMemsetAsync(A.ob.nFallback, 0, sizeof(int), st);
   launch_chain_counts(k.headCap, &C->nHeads, A.heads, A.sb, A.mb, A.trkNcl, st);
   scan_exclusive(A.trkNcl, A.ob.off, k.headCap, &C->nHeads, A.scratch, st);
-  launch_final_refit(k.headCap, &C->nHeads, A.heads, A.sb, A.mb, A.syz, A.sorig, A.tfs, G, forceFp64, A.ob, st);
+  launch_final_refit(k.headCap, &C->nHeads, k.stCap, A.heads, A.sb, A.mb, A.syz, A.tfs, G, forceFp64,
+                     A.workCounter + 5, A.perm, A.ob, st);
   launch_lower_bounds(A.heads, &C->nHeads, A.stTfBegin, k.BCap + 1, A.trkTfBegin, st);
   // continuous readout
   MergeBufs mm = A.mb;

@@ -37,6 +37,7 @@ struct GraphArena {
   int* tlTfBegin;
   TrackletBufs tb;
   int* workCounter;
+  int* perm;  // processing order of the passes
   unsigned long long* w;
   int *secBegin, *wide, *nSeg, *nSegHits, *segPos, *segHitPos;
   SectorTrackBufs sb;
@@ -45,7 +46,6 @@ struct GraphArena {
   int *headFlag, *heads, *trkNcl;
   OutBufs ob;
   OutBufs ob2;  // a second set of result arrays: replays alternate between the two
-  int *lenHist, *stOrder;  // the sector fits' longest-first processing order
   int* trkTfBegin;
   double* coll;                       // interaction times of the batch
   int *memNext, *memPrev, *memPairs;  // membrane links and their pair count

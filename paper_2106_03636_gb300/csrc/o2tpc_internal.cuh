@@ -211,6 +211,20 @@ __device__ inline int upper_bound_i32(const int* a, int n, int v) {
   return lo;
 }
 
+// ---------------------------------------------- work in order of length
+// Persistent warps: the next 32 of n items, in the order perm (see
+// launch_length_order); item: this lane's, -1 if there is none for it.  False
+// when no items are left.  All lanes call it.
+__device__ inline bool take_ordered(int* counter, const int* __restrict__ perm, int n, int& item) {
+  const int lane = threadIdx.x & 31;
+  int j = 0;
+  if (lane == 0) j = atomicAdd(counter, 32);
+  j = __shfl_sync(0xffffffffu, j, 0);
+  if (j >= n) return false;
+  item = j + lane < n ? perm[j + lane] : -1;
+  return true;
+}
+
 // ------------------------------------------------- Kalman building blocks
 // State (y, zeta, sin phi, t = dzeta/ds_T, q/pT) at local x; covariance as
 // lower triangle (yy, zy, zz, sy, sz, ss, ty, tz, ts, tt, qy, qz, qs, qt, qq).

@@ -65,12 +65,12 @@ void launch_clean(int n, const int* nDev, const int* upRaw, const int* dnRaw, in
                   cudaStream_t st);
 int scan_scratch_ints(long long n);
 void scan_exclusive(const int* in, int* out, int n, const int* nDev, int* scratch, cudaStream_t st);
-// perm[0, m) = 0..m-1 (m = *nDev <= n) ordered by descending length
-// off[i + 1] - off[i] (lengths clamped to kLenBins - 1; any order among equal
-// lengths), so that a kernel walking perm with one thread per item gives the
-// 32 lanes of a warp items of about equal length.  hist: kLenBins ints.
-constexpr int kLenBins = 512;
-void launch_len_order(int n, const int* nDev, const int* off, int* hist, int* perm, cudaStream_t st);
+// perm[0, m) = 0..m-1 (m = *nDev <= n), every 1024 consecutive items longest
+// first; lengths a[i], or a[i + 1] - a[i] with diff (clamped to 255; any order
+// among equals).  Kernels with one thread per item whose cost goes with its
+// length walk perm: the 32 lanes of a warp then have items of about equal
+// length, and the items' data still lie together in memory.
+void launch_length_order(int n, const int* nDev, const int* a, bool diff, int* perm, cudaStream_t st);
 // Ordered compaction with warp ballots: the indices i < *nDev with flag[i]
 // set, ascending, into out (at most cap; more raise *overflow).
 // launch_ballot_count: tile counts, their scan into tileOff and *count;
@@ -111,10 +111,13 @@ struct TrackletBufs {
 // drift-ordered views (identical results).  keepState: leave the whole state
 // in tb.state; without it the inward pass leaves x and the three direction
 // parameters, which is all the sector fits read.
-// nTl sizes the grids; the kernels read the count at nTlDev
+// nTl sizes the grids; the kernels read the count at nTlDev.  workCounter:
+// kWorkCounters ints, zeroed here (also without tracklets): the four passes',
+// then the sector fits' and the final refit's.
+constexpr int kWorkCounters = 6;
 void launch_tracklets(int nTl, const int* nTlDev, int* workCounter, const int* starts, const int* up,
                       const RowGrid* grid, int nRows, const int* cellStart, const int2* syz, const GeomConst* G,
-                      ZView zv, TrackletBufs tb, cudaStream_t st, cudaEvent_t* passEnd = nullptr,
+                      ZView zv, TrackletBufs tb, int* perm, cudaStream_t st, cudaEvent_t* passEnd = nullptr,
                       bool coopSearch = false, bool keepState = false);
 
 struct SectorTrackBufs {
@@ -143,14 +146,16 @@ void launch_segments_write(int nTl, const int* nTlDev, const int* secBegin, cons
 // sb.yz / sb.orig of every sector-track hit (after the CSR end is written)
 void launch_st_gather(int nHits, const int* nHitsDev, SectorTrackBufs sb, const int2* syz, const int* sorig,
                       cudaStream_t st);
-// order: the sector tracks in the order the fits take them (launch_len_order of sb.off)
-void launch_sector_fit(int nSt, const int* nStDev, const TrackletBufs tb, const int2* syz, const GeomConst* G,
-                       SectorTrackBufs sb, const int* order, cudaStream_t st);
+// perm (here, in the tracklet passes and in the final refit): scratch for the
+// processing order, one int per item; counter: a zeroed work counter.
+void launch_sector_fit(int nSt, const int* nStDev, int* counter, int* perm, const TrackletBufs tb, const GeomConst* G,
+                       SectorTrackBufs sb, cudaStream_t st);
 
 // k_merge.cu
 struct MergeBufs {
-  int* keyIn;        // [nSt] B-list key of the inner end (-1: not a border end)
-  int* keyOut;       // [nSt] edge key of the outer end (-1)
+  int* keyIn;        // [nSt] B-list key of the inner end (-1: not a border end); from the chain counts
+                     // on the segment's track (-1: none)
+  int* keyOut;       // [nSt] edge key of the outer end (-1); then the segment's first place in the track
   int* listCnt;      // [nKeys + 1]
   int* listStart;    // [nKeys + 1]
   int* listItems;    // [nSt]
@@ -207,9 +212,10 @@ struct OutBufs {
   int* mate;        // track linked across the central membrane, or -1
   int* coll;        // interaction time index inside the TF, or -1
 };
-void launch_final_refit(int nHeads, const int* nHeadsDev, const int* heads, const SectorTrackBufs sb, MergeBufs mb,
-                        const int2* syz, const int* sorig, const TFDesc* tfs, const GeomConst* G, int forceFp64,
-                        OutBufs ob, cudaStream_t st);
+// (after launch_chain_counts, whose segment places it reads in mb.keyIn / keyOut)
+void launch_final_refit(int nHeads, const int* nHeadsDev, int nSt, const int* heads, const SectorTrackBufs sb,
+                        MergeBufs mb, const int2* syz, const TFDesc* tfs, const GeomConst* G, int forceFp64,
+                        int* counter, int* perm, OutBufs ob, cudaStream_t st);
 // Compressed TF (csrc/k_ctf.cu).  Stream table entry: first symbol, symbol
 // count, first chunk, chunk count.
 struct CtfStream {
