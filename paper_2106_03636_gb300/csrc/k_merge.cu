@@ -582,13 +582,184 @@ __global__ void __launch_bounds__(128) k_final_refit(const int* __restrict__ nHe
   }
 }
 
+// ---- the FP64 refit of one track by one warp
+// Lane 5 i + j (below 25) holds element (i, j) of the symmetric covariance;
+// lane 5 i also the parameter i.  Per hit a warp issues ~50 double-precision
+// instructions where a thread working through all elements issues ~180; a
+// GB300 runs one per 64 cycles and SM quarter, so a handful of tracks (the
+// usual case: 1-5 of a Time Frame) take the time of their longest chain of
+// them.
+struct Refit64 {
+  int i, j, ii, jj;  // element, and the same with ii >= jj
+  double c, p;       // covariance element; parameter of row i
+};
+__device__ inline double lane_of(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+// Element (max, min) of two indices of a symmetric matrix held per lane.
+__device__ inline double elem(double v, int a, int b) { return lane_of(v, 5 * max(a, b) + min(a, b)); }
+
+// C <- J C J^T for the transport Jacobian (as kf_sandwich_transport).
+__device__ inline void transport64(Refit64& t, const PropStep<float>& o) {
+  const double a02 = o.a02, a04 = o.a04, a12 = o.a12, a13 = o.a13, a14 = o.a14, a24 = o.a24;
+  const double c2 = lane_of(t.c, 10 + t.j), c3 = lane_of(t.c, 15 + t.j), c4 = lane_of(t.c, 20 + t.j);
+  const double f2 = t.i == 0 ? a02 : t.i == 1 ? a12 : 0.0, f3 = t.i == 1 ? a13 : 0.0;
+  const double f4 = t.i == 0 ? a04 : t.i == 1 ? a14 : t.i == 2 ? a24 : 0.0;
+  const double m = t.c + f2 * c2 + f3 * c3 + f4 * c4;  // (J C)(i, j)
+  const double m0 = lane_of(m, 5 * t.ii + t.jj), m2 = lane_of(m, 5 * t.ii + 2), m3 = lane_of(m, 5 * t.ii + 3),
+               m4 = lane_of(m, 5 * t.ii + 4);
+  const double g2 = t.jj == 0 ? a02 : t.jj == 1 ? a12 : 0.0, g3 = t.jj == 1 ? a13 : 0.0;
+  const double g4 = t.jj == 0 ? a04 : t.jj == 1 ? a14 : t.jj == 2 ? a24 : 0.0;
+  t.c = m0 + g2 * m2 + g3 * m3 + g4 * m4;
+}
+
+// Frame rotation (as kf_rotate); x and y are absolute.
+__device__ inline int rotate64(Refit64& t, double& x, double ca, double sa, double bzc) {
+  const double sp = lane_of(t.p, 10), tl = lane_of(t.p, 15), q = lane_of(t.p, 20), y = lane_of(t.p, 0);
+  if (fabs(sp) >= (double)kSinProp) return -1;
+  const double c = sqrt((1.0 - sp) * (1.0 + sp));
+  const double s2 = sp * ca - c * sa, c2 = c * ca + sp * sa;
+  if (c2 <= 0.0 || fabs(s2) >= (double)kSinProp) return -1;
+  const double J00 = c / c2, J10 = -tl * sa / c2, J20 = -q * bzc * sa, J22 = c2 / c;
+  // A = J C, then s = A J^T and the mean with its transpose
+  const double m0 = lane_of(t.c, t.j);
+  const double a = t.i == 0 ? J00 * m0 : t.i == 1 ? J10 * m0 + t.c : t.i == 2 ? J20 * m0 + J22 * t.c : t.c;
+  const double a0 = lane_of(a, 5 * t.i);
+  const double s = t.j == 0 ? a0 * J00 : t.j == 1 ? a0 * J10 + a : t.j == 2 ? a0 * J20 + a * J22 : a;
+  t.c = 0.5 * (s + lane_of(s, 5 * t.j + t.i));
+  if (t.i == 0) t.p = -x * sa + y * ca;
+  if (t.i == 2) t.p = s2;
+  x = x * ca + y * sa;
+  return 0;
+}
+
+// refit_chain<double> with the state spread over the warp; all lanes return
+// the same flags, chi2, used and frame.
+__device__ int refit_chain64(int head, int tail, const SectorTrackBufs& sb, const int* __restrict__ prev,
+                             const GeomConst* __restrict__ G, int zref, Refit64& t, double& x, double& chi2,
+                             int& used, int& frame, int* yrefOut) {
+  const double zunit = G->zunit_d, bzc = G->bzc_d, yunit = 1.0 / 160.0;
+  const int angErr = G->angErr;
+  frame = sb.sector[tail];
+  const int hl = sb.off[tail + 1] - 1;
+  const float* so = sb.out + (size_t)tail * 21;
+  const int2 pl = sb.yz[hl];
+  int yref = pl.x, zcur = pl.y, srow = sb.rows[hl];
+  x = G->rowx_d[srow];
+  t.p = t.i >= 2 ? (double)so[1 + t.i] : 0.0;
+  double vy, vz;
+  auto variances = [&]() {  // cluster variances at the state's angles
+    KState<double> s;
+    s.p[2] = lane_of(t.p, 10);
+    s.p[3] = lane_of(t.p, 15);
+    meas_var<double>(angErr, s, vy, vz);
+  };
+  variances();
+  t.c = t.i != t.j ? 0.0 : t.i == 0 ? vy : t.i == 1 ? vz : t.i == 2 ? 0.04 : t.i == 3 ? 0.25 : 400.0;
+  chi2 = 0.0;
+  used = 1;
+  bool first = true;
+  for (int sg = tail;; sg = prev[sg]) {
+    const int sec = sb.sector[sg];
+    for (int h = sb.off[sg + 1] - 1; h >= sb.off[sg]; --h) {
+      if (first) { first = false; continue; }
+      const int2 p = sb.yz[h];
+      if (sec != frame) {
+        const int dd = ((sec % 18) - (frame % 18) + 18) % 18;
+        const double sgn = (dd == 1) ? 1.0 : -1.0;
+        if (t.i == 0) t.p += (double)yref * yunit;
+        if (rotate64(t, x, G->rot_cos_d, sgn * G->rot_sin_d, bzc) != 0) {
+          if (t.i == 0) t.p -= (double)yref * yunit;
+          if (t.i == 1) t.p += (double)(zcur - zref) * zunit;
+          *yrefOut = yref;
+          return 4;
+        }
+        yref = p.x;
+        if (t.i == 0) t.p -= (double)yref * yunit;
+        frame = sec;
+        srow = -1;
+      }
+      const int ri = sb.rows[h];
+      const float dx = srow >= 0 ? (float)(ri - srow) * G->pitch : (float)(G->rowx_d[ri] - x);
+      if (dx != 0.f) {  // the step's geometry in single precision, as kf_prop_dx_cov64
+        const double q = lane_of(t.p, 20);
+        const float pf[5] = {0.f, 0.f, (float)lane_of(t.p, 10), (float)lane_of(t.p, 15), (float)q};
+        PropStep<float> o;
+        if (kf_prop_step<float, kF1Rounded>(pf, dx, G->bzc, o) != 0) continue;
+        if (t.i == 0) t.p += (double)o.dy;
+        if (t.i == 1) t.p += (double)o.dzeta;
+        if (t.i == 2) t.p += q * (double)G->bzc * (double)dx;
+        x = G->rowx_d[ri];
+        transport64(t, o);
+      }
+      srow = ri;
+      const int m = floordiv_i32(p.x - yref + 80, 160);
+      yref += 160 * m;
+      if (t.i == 0 && m != 0) t.p -= (double)m;
+      if (t.i == 1 && p.y != zcur) t.p -= (double)(p.y - zcur) * zunit;
+      zcur = p.y;
+      // update
+      variances();
+      const double r0 = (double)(p.x - yref) * yunit - lane_of(t.p, 0), r1 = 0.0 - lane_of(t.p, 5);
+      const double S01 = elem(t.c, 1, 0), S00 = lane_of(t.c, 0) + vy, S11 = lane_of(t.c, 6) + vz;
+      const double det = S00 * S11 - S01 * S01;
+      if (!(det > 0.0)) continue;
+      const double idet = 1.0 / det;
+      const double I00 = S11 * idet, I01 = -S01 * idet, I11 = S00 * idet;
+      chi2 += r0 * r0 * I00 + 2.0 * r0 * r1 * I01 + r1 * r1 * I11;
+      const double cyi = lane_of(t.c, 5 * t.ii), czi = lane_of(t.c, 5 * t.ii + 1);
+      const double cyj = lane_of(t.c, 5 * t.jj), czj = lane_of(t.c, 5 * t.jj + 1);
+      const double K0 = cyi * I00 + czi * I01, K1 = cyi * I01 + czi * I11;
+      if (t.j == 0) t.p += K0 * r0 + K1 * r1;  // there ii = i
+      t.c -= K0 * cyj + K1 * czj;
+      ++used;
+    }
+    if (sg == head) break;
+  }
+  if (t.i == 1) t.p += (double)(zcur - zref) * zunit;  // zeta back to the track's origin
+  *yrefOut = yref;
+  return 0;
+}
+
 // K11b: the queued tracks again with an FP64 covariance (flag bit 1): the
 // state and its covariance in double, each transport step's geometry in
-// single precision (kf_prop_dx_cov64).
+// single precision (kf_prop_dx_cov64).  Up to kWarpRefit64 tracks a warp each,
+// more a thread each: 608 SM quarters share the tracks, and a warp's step costs
+// ~50 instructions for one track against ~180 for 32, so the lines cross at
+// about 608 * 180 / 50.
+// One track of the 1 ms frame: 0.94 -> 0.36 ms; four of 32 orbits 0.49 -> 0.18.
+constexpr int kWarpRefit64 = 2048;
 __global__ void __launch_bounds__(128) k_final_refit64(const int* __restrict__ heads, SectorTrackBufs sb, MergeBufs mb,
                                                        const int2* __restrict__ syz, const GeomConst* __restrict__ G,
                                                        OutBufs ob) {
   const int nf = *ob.nFallback;
+  if (nf <= kWarpRefit64) {
+    const int lane = threadIdx.x & 31;
+    Refit64 r;
+    r.i = min(lane / 5, 4);
+    r.j = lane < 25 ? lane % 5 : 4;
+    r.ii = max(r.i, r.j);
+    r.jj = min(r.i, r.j);
+    // warps of one block come last: neighbours in the queue go to different SMs
+    for (int q = blockIdx.x + gridDim.x * (threadIdx.x >> 5); q < nf; q += gridDim.x * (blockDim.x >> 5)) {
+      const int t = ob.fallback[q];
+      const int head = heads[t];
+      int nseg;
+      const int tail = chain_tail(head, mb.next, &nseg);
+      const int zref = sb.yz[sb.off[head]].y;
+      KState<double> sd;
+      double c2d;
+      int used, frame, yref;
+      const int fl = refit_chain64(head, tail, sb, mb.prev, G, zref, r, sd.x, c2d, used, frame, &yref);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sd.p[k] = lane_of(r.p, 5 * k);
+#pragma unroll
+      for (int a = 0; a < 5; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b) sd.C[ix(a, b)] = lane_of(r.c, 5 * a + b);
+      if (lane == 0)
+        write_track<double>(t, sd, yref, c2d, used, frame, 1 | (nseg > 1 ? 2 : 0) | (fl & 4), zref, G, ob);
+    }
+    return;
+  }
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nf; q += gridDim.x * blockDim.x) {
     const int t = ob.fallback[q];
     const int head = heads[t];

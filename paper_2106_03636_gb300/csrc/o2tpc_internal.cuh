@@ -441,7 +441,7 @@ __device__ inline int kf_prop_dx_cov64(KState<double>& s, double x2, float dx, f
 #pragma unroll
   for (int i = 0; i < 5; ++i) pf[i] = (float)s.p[i];
   PropStep<float> o;
-  if (kf_prop_step<float>(pf, dx, bzc, o) != 0) return -1;
+  if (kf_prop_step<float, kF1Rounded>(pf, dx, bzc, o) != 0) return -1;
   s.p[0] += (double)o.dy;
   s.p[1] += (double)o.dzeta;
   s.p[2] += s.p[4] * (double)bzc * (double)dx;
