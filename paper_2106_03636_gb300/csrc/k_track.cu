@@ -767,24 +767,6 @@ __device__ inline void load_hits8(const int* H, int (&hh)[8]) {
   hh[4] = b.x; hh[5] = b.y; hh[6] = b.z; hh[7] = b.w;
 }
 
-// Ownership bits of slots [0, nh) of a tracklet into this thread's column of
-// own[5][128] (bit i % 32 of word i / 32 set: slot i's hit is owned by it).
-__device__ inline void owned_bits(const OwnCtx& o, const TlKey& key, const int* H, int nh, unsigned (*own)[128]) {
-  for (int i = 0; i < nh; i += 8) {
-    int hh[8];
-    load_hits8(H + i, hh);
-    bool ok[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) ok[u] = (i + u < nh) && key.owns(o, hh[u]);
-    unsigned bits = 0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) bits |= (unsigned)ok[u] << u;
-    if ((i & 31) == 0) own[i >> 5][threadIdx.x] = bits;
-    else own[i >> 5][threadIdx.x] |= bits << (i & 31);
-  }
-}
-__device__ inline bool is_owned(const unsigned (*own)[128], int i) { return (own[i >> 5][threadIdx.x] >> (i & 31)) & 1u; }
-
 // K8a: hit ownership (atomicMax of the key; a hit already holding a larger
 // key is skipped without an atomic).
 __global__ void k_ownership(const int* __restrict__ nTlDev, OwnCtx o, TrackletBufs tb) {
@@ -819,105 +801,252 @@ __global__ void k_ownership(const int* __restrict__ nTlDev, OwnCtx o, TrackletBu
   }
 }
 
-// K8b: segments per tracklet (count pass): owned hits in row order, split at
-// gaps of more than kMaxMiss rows, segments of >= kMinHits kept.
-__global__ void __launch_bounds__(128) k_segments_count(const int* __restrict__ nTlDev, OwnCtx o, TrackletBufs tb,
-                                                        int* __restrict__ nSeg, int* __restrict__ nSegHits) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= *nTlDev) return;
-  __shared__ unsigned s_own[(kMaxTlHits + 31) / 32][128];
-  const int nh = tb.nhits[k];
-  int cs = 0, ch = 0;
-  if (nh >= kMinHits) {
-    const TlKey key = tl_key(o, tb, k, nh);
-    const int nasc = tb.nasc[k], nd = nh - nasc;
-    const int* H = tb.hits + (size_t)k * kMaxTlHits;
-    const uint8_t* Rw = tb.rows + (size_t)k * kMaxTlHits;
-    owned_bits(o, key, H, nh, s_own);
-    int m = 0, prev = -1000;
-    for (int j = 0; j < nh; ++j) {
-      const int i = (j < nd) ? (nh - 1 - j) : (j - nd);
-      if (!is_owned(s_own, i)) continue;
-      const int row = Rw[i];
-      if (m > 0 && row - prev - 1 > kMaxMiss) {
-        if (m >= kMinHits) { ++cs; ch += m; }
-        m = 0;
-      }
-      ++m;
-      prev = row;
-    }
-    if (m >= kMinHits) { ++cs; ch += m; }
-  }
-  nSeg[k] = cs;
-  nSegHits[k] = ch;
+// Segments: a tracklet's owned hits in row order (its inward hits backwards,
+// then its chain and outward hits), split at gaps of more than kMaxMiss rows;
+// segments of >= kMinHits are kept.  A warp takes a group of consecutive
+// tracklets, loads what it needs of each at once, and works on one after the
+// other with a lane per hit, the next one's lists on their way: lists, rows and
+// results are read and written as whole lines, 32 random words in flight.
+// (With a thread per tracklet the write pass ran with 6.5 of 32 lanes active.)
+// 1 ms frame: count 0.30 -> 0.31, write with the coordinate gather 0.55 -> 0.32
+// ms; one sector's frame 39 + 57 -> 8 + 8 us; 32 orbits 0.76 + 1.44 -> 0.95 + 1.35.
+constexpr int kSegWords = kOwnWords;
+
+// Slot of the tracklet's j-th hit in row order (nd of its nh hits are inward).
+__device__ inline int slot_of(int j, int nh, int nd) { return j < nd ? nh - 1 - j : j - nd; }
+
+// Of the owned hits `own` of 32 consecutive places (lane = place): those that
+// begin a segment.  prevRow: row of the last owned hit before (a large negative
+// number if there is none), moved on.
+__device__ inline unsigned segment_starts(unsigned own, int row, int& prevRow) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const unsigned before = own & ((1u << lane) - 1u);
+  const int pl = __shfl_sync(full, row, before ? 31 - __clz(before) : 0);
+  const int pr = before ? pl : prevRow;
+  const unsigned st = __ballot_sync(full, ((own >> lane) & 1u) && row - pr - 1 > kMaxMiss);
+  if (own) prevRow = __shfl_sync(full, row, 31 - __clz(own));
+  return st;
 }
 
-// K8c: write the sector tracks of each tracklet (ids in tracklet order).
-// Hits go straight to their output slots: a segment that turns out too short
-// is overwritten by the next kept one, or lies past the tracklet's last kept
-// hit and is not written (the slots of a tracklet are exactly its kept hits).
-__global__ void __launch_bounds__(128) k_segments_write(const int* __restrict__ nTlDev, OwnCtx o, TrackletBufs tb,
+// A tracklet's hits and rows in row order, five places a lane.
+struct TlPlaces {
+  int hit[kSegWords], row[kSegWords];
+  __device__ void load(const TrackletBufs& tb, int k, int nh, int nd) {
+    const int lane = threadIdx.x & 31;
+    const int* H = tb.hits + (size_t)k * kMaxTlHits;
+    const uint8_t* Rw = tb.rows + (size_t)k * kMaxTlHits;
+#pragma unroll
+    for (int c = 0; c < kSegWords; ++c) {
+      const int j = c * 32 + lane;
+      hit[c] = -1;
+      row[c] = 0;
+      if (j < nh) {
+        const int i = slot_of(j, nh, nd);
+        hit[c] = H[i];
+        row[c] = Rw[i];
+      }
+    }
+  }
+};
+
+// Consecutive tracklets a warp takes at once: 32, fewer when there are too few
+// for every warp of the grid.
+__device__ inline int segment_group(int nTl) {
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  return min(32, max(1, (nTl + warps - 1) / warps));
+}
+
+// K8b: count pass; also keeps the ownership bits (in row order) for the write
+// pass, which then reads no ownership words.
+__global__ void __launch_bounds__(128, 10) k_segments_count(const int* __restrict__ nTlDev, OwnCtx o, TrackletBufs tb,
+                                                        int* __restrict__ nSeg, int* __restrict__ nSegHits,
+                                                        unsigned* __restrict__ ownBits) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, nTl = *nTlDev;
+  const int group = segment_group(nTl), warps = gridDim.x * (blockDim.x >> 5);
+  const bool wide = *o.wide != 0;
+  for (int k0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * group; k0 < nTl; k0 += warps * group) {
+    const int kl = k0 + lane;
+    const bool mineTl = lane < group && kl < nTl;
+    // of this lane's tracklet
+    const int nhl = mineTl ? tb.nhits[kl] : 0;
+    int ndl = 0, lidl = 0;
+    if (nhl >= kMinHits) {
+      ndl = nhl - tb.nasc[kl];
+      lidl = kl - o.secBegin[tb.rbase[kl] / kNRow];
+    }
+    int csl = 0, chl = 0;
+    unsigned todo = __ballot_sync(full, nhl >= kMinHits);
+    TlPlaces next;
+    auto fetch = [&]() {
+      const int src = todo ? __ffs(todo) - 1 : 0;
+      const int nh = __shfl_sync(full, nhl, src), nd = __shfl_sync(full, ndl, src);
+      if (todo) next.load(tb, k0 + src, nh, nd);
+    };
+    fetch();
+    while (todo) {
+      const int src = __ffs(todo) - 1, k = k0 + src;
+      todo &= todo - 1;
+      const TlPlaces T = next;
+      const int nh = __shfl_sync(full, nhl, src), lid = __shfl_sync(full, lidl, src);
+      bool mine[kSegWords];
+      if (wide) {
+        const unsigned long long key = own_key64(nh, lid);
+#pragma unroll
+        for (int c = 0; c < kSegWords; ++c)
+          mine[c] = T.hit[c] >= 0 && static_cast<const unsigned long long*>(o.w)[T.hit[c]] == key;
+      } else {
+        const unsigned key = own_key32(nh, lid);
+#pragma unroll
+        for (int c = 0; c < kSegWords; ++c)
+          mine[c] = T.hit[c] >= 0 && static_cast<const unsigned*>(o.w)[T.hit[c]] == key;
+      }
+      fetch();
+      int cs = 0, ch = 0, m = 0, prevRow = -1000;
+#pragma unroll
+      for (int c = 0; c < kSegWords; ++c) {
+        const unsigned own = __ballot_sync(full, mine[c]);
+        if (lane == c) ownBits[(size_t)k * kSegWords + c] = own;
+        if (!own) continue;
+        unsigned rest = own;
+        for (unsigned st = segment_starts(own, T.row[c], prevRow); st; st &= st - 1) {
+          const unsigned lower = (st & -st) - 1u;  // places before the start
+          m += __popc(rest & lower);
+          if (m >= kMinHits) {
+            ++cs;
+            ch += m;
+          }
+          m = 0;
+          rest &= ~lower;
+        }
+        m += __popc(rest);
+      }
+      if (m >= kMinHits) {
+        ++cs;
+        ch += m;
+      }
+      if (lane == src) {
+        csl = cs;
+        chl = ch;
+      }
+    }
+    if (mineTl) {
+      nSeg[kl] = csl;
+      nSegHits[kl] = chl;
+    }
+  }
+}
+
+// K8c: write the sector tracks of each tracklet (ids in tracklet order) and
+// gather the coordinates and input indices of their hits for the fits.  A
+// tracklet has at most 27 segments, kept or not (they lie 6 rows apart): a lane
+// each for their table entries.
+__global__ void __launch_bounds__(128, 6) k_segments_write(const int* __restrict__ nTlDev, TrackletBufs tb,
+                                                        const unsigned* __restrict__ ownBits,
                                                         const int* __restrict__ segPos,
                                                         const int* __restrict__ segHitPos,
                                                         const int2* __restrict__ syz,
                                                         const int* __restrict__ sorig, SectorTrackBufs sb, int capSt,
                                                         int capHits) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= *nTlDev) return;
-  const int nh = tb.nhits[k];
-  if (nh < kMinHits || segPos[k + 1] == segPos[k]) return;
-  __shared__ unsigned s_own[(kMaxTlHits + 31) / 32][128];
-  const TlKey key = tl_key(o, tb, k, nh);
-  const int nasc = tb.nasc[k], nd = nh - nasc;
-  const int* H = tb.hits + (size_t)k * kMaxTlHits;
-  const uint8_t* Rw = tb.rows + (size_t)k * kMaxTlHits;
-  owned_bits(o, key, H, nh, s_own);
-  const int ts = tb.rbase[k] / kNRow;
-  const int tf = ts / kNSec, sector = ts % kNSec;
-  // the slots end at the tracklet's last kept hit, and at the capacity
-  const int hoEnd = min(segHitPos[k + 1], capHits);
-  int id = segPos[k], ho = segHitPos[k];
-  int m = 0, prev = -1000, first = -1;
-  auto flush = [&](void) {
-    if (m >= kMinHits) {
-      if (id < capSt) {
-        sb.tl[id] = k;
-        sb.tf[id] = tf;
-        sb.sector[id] = sector;
-        sb.off[id] = min(ho, capHits);
-        sb.zref[id] = syz[first].y;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, nTl = *nTlDev;
+  const int group = segment_group(nTl), warps = gridDim.x * (blockDim.x >> 5);
+  for (int k0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * group; k0 < nTl; k0 += warps * group) {
+    const int kl = k0 + lane;
+    const bool mineTl = lane < group && kl < nTl;
+    const int idl = mineTl ? segPos[kl] : 0;
+    const bool some = mineTl && segPos[kl + 1] > idl;
+    int nhl = 0, ndl = 0, tsl = 0, hol = 0;
+    unsigned ownl[kSegWords] = {};
+    if (some) {
+      nhl = tb.nhits[kl];
+      ndl = nhl - tb.nasc[kl];
+      tsl = tb.rbase[kl] / kNRow;
+      hol = segHitPos[kl];
+#pragma unroll
+      for (int c = 0; c < kSegWords; ++c) ownl[c] = ownBits[(size_t)kl * kSegWords + c];
+    }
+    unsigned todo = __ballot_sync(full, some);
+    TlPlaces next;
+    auto fetch = [&]() {
+      const int src = todo ? __ffs(todo) - 1 : 0;
+      const int nh = __shfl_sync(full, nhl, src), nd = __shfl_sync(full, ndl, src);
+      if (todo) next.load(tb, k0 + src, nh, nd);
+    };
+    fetch();
+    while (todo) {
+      const int src = __ffs(todo) - 1, k = k0 + src;
+      todo &= todo - 1;
+      const TlPlaces T = next;
+      unsigned own[kSegWords];
+      int2 yz[kSegWords];
+      int orig[kSegWords];
+#pragma unroll
+      for (int c = 0; c < kSegWords; ++c) {
+        own[c] = __shfl_sync(full, ownl[c], src);
+        if ((own[c] >> lane) & 1u) {
+          yz[c] = syz[T.hit[c]];
+          orig[c] = sorig[T.hit[c]];
+        }
       }
-      ++id;
-      ho += m;
+      fetch();
+      // lane q: hits of segment q and owned hits before it
+      unsigned start[kSegWords];
+      int seg = -1, total = 0, prevRow = -1000, rankl = 0;
+#pragma unroll
+      for (int c = 0; c < kSegWords; ++c) {
+        start[c] = own[c] ? segment_starts(own[c], T.row[c], prevRow) : 0u;
+        for (unsigned st = start[c]; st; st &= st - 1) {
+          ++seg;
+          const int before = total + __popc(own[c] & ((st & -st) - 1u));
+          if (lane == seg) rankl = before;
+        }
+        total += __popc(own[c]);
+      }
+      const int nextRank = __shfl_down_sync(full, rankl, 1);
+      const int len = lane > seg ? 0 : (lane == seg ? total : nextRank) - rankl;
+      const bool keep = len >= kMinHits;
+      const unsigned kept = __ballot_sync(full, keep);
+      // output slots of the kept ones and their table entries
+      int ho = keep ? len : 0;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(full, ho, d);
+        if (lane >= d) ho += y;
+      }
+      ho += __shfl_sync(full, hol, src) - (keep ? len : 0);
+      const int ts = __shfl_sync(full, tsl, src);
+      const int id = __shfl_sync(full, idl, src) + __popc(kept & ((1u << lane) - 1u));
+      if (keep && id < capSt) {
+        sb.tl[id] = k;
+        sb.tf[id] = ts / kNSec;
+        sb.sector[id] = ts % kNSec;
+        sb.off[id] = min(ho, capHits);
+      }
+      // the hits: a place's segment is the last one that starts at or before it
+      int segBefore = -1, rankBefore = 0;
+#pragma unroll
+      for (int c = 0; c < kSegWords; ++c) {
+        const unsigned below = (1u << lane) - 1u;
+        const int q = max(segBefore + __popc(start[c] & (below | (1u << lane))), 0);
+        const int dst = __shfl_sync(full, ho, q), first = __shfl_sync(full, rankl, q), idq = __shfl_sync(full, id, q);
+        const int r = rankBefore + __popc(own[c] & below) - first;  // place in the segment
+        if (((own[c] >> lane) & 1u) && ((kept >> q) & 1u)) {
+          const int at = dst + r;
+          if (at < capHits) {
+            sb.hits[at] = T.hit[c];
+            sb.rows[at] = (uint8_t)T.row[c];
+            sb.yz[at] = yz[c];
+            sb.orig[at] = orig[c];
+          }
+          if (r == 0 && idq < capSt) sb.zref[idq] = yz[c].y;
+        }
+        segBefore += __popc(start[c]);
+        rankBefore += __popc(own[c]);
+      }
     }
-    m = 0;
-  };
-  for (int j = 0; j < nh; ++j) {
-    const int i = (j < nd) ? (nh - 1 - j) : (j - nd);
-    if (!is_owned(s_own, i)) continue;
-    const int h = H[i];
-    const int row = Rw[i];
-    if (m > 0 && row - prev - 1 > kMaxMiss) flush();
-    if (m == 0) first = h;
-    if (ho + m < hoEnd) {
-      sb.hits[ho + m] = h;
-      sb.rows[ho + m] = (uint8_t)row;
-    }
-    ++m;
-    prev = row;
   }
-  flush();
-}
-
-// K8d: coordinates and input index of every sector-track hit, gathered once
-// (one thread per hit) for the sector fits and the final refit.
-__global__ void k_st_gather(const int* __restrict__ nHitsDev, SectorTrackBufs sb, const int2* __restrict__ syz,
-                            const int* __restrict__ sorig) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= *nHitsDev) return;
-  const int h = sb.hits[i];
-  sb.yz[i] = syz[h];
-  sb.orig[i] = sorig[h];
 }
 
 // The sector tracks' fits, one thread per track, the tracks in order of
@@ -1060,29 +1189,26 @@ void launch_ownership(int nTl, const int* nTlDev, int nSec, const RowGrid* grid,
   }
 }
 
+namespace {
+// warps of 1 to 32 tracklets, up to twelve blocks of four warps an SM
+int segment_blocks(int nTl) { return std::min((nTl + 3) / 4, pass_grid().sms * 12); }
+}  // namespace
+
 void launch_segments_count(int nTl, const int* nTlDev, const int* secBegin, const int* wide, const void* w,
-                           TrackletBufs tb, int* nSeg, int* nSegHits, cudaStream_t st) {
+                           TrackletBufs tb, int* nSeg, int* nSegHits, unsigned* ownBits, cudaStream_t st) {
   if (nTl > 0) {
-    k_segments_count<<<(nTl + 127) / 128, 128, 0, st>>>(nTlDev, OwnCtx{secBegin, wide, const_cast<void*>(w)}, tb,
-                                                         nSeg, nSegHits);
+    k_segments_count<<<segment_blocks(nTl), 128, 0, st>>>(nTlDev, OwnCtx{secBegin, wide, const_cast<void*>(w)}, tb,
+                                                          nSeg, nSegHits, ownBits);
     ++g_launch_count;
   }
 }
 
-void launch_segments_write(int nTl, const int* nTlDev, const int* secBegin, const int* wide, const void* w,
-                           TrackletBufs tb, const int* segPos, const int* segHitPos, const int2* syz,
-                           const int* sorig, SectorTrackBufs sb, int capSt, int capHits, cudaStream_t st) {
+void launch_segments_write(int nTl, const int* nTlDev, TrackletBufs tb, const unsigned* ownBits, const int* segPos,
+                           const int* segHitPos, const int2* syz, const int* sorig, SectorTrackBufs sb, int capSt,
+                           int capHits, cudaStream_t st) {
   if (nTl > 0) {
-    k_segments_write<<<(nTl + 127) / 128, 128, 0, st>>>(nTlDev, OwnCtx{secBegin, wide, const_cast<void*>(w)}, tb,
-                                                         segPos, segHitPos, syz, sorig, sb, capSt, capHits);
-    ++g_launch_count;
-  }
-}
-
-void launch_st_gather(int nHits, const int* nHitsDev, SectorTrackBufs sb, const int2* syz, const int* sorig,
-                      cudaStream_t st) {
-  if (nHits > 0) {
-    k_st_gather<<<(nHits + 255) / 256, 256, 0, st>>>(nHitsDev, sb, syz, sorig);
+    k_segments_write<<<segment_blocks(nTl), 128, 0, st>>>(nTlDev, tb, ownBits, segPos, segHitPos, syz, sorig, sb,
+                                                          capSt, capHits);
     ++g_launch_count;
   }
 }

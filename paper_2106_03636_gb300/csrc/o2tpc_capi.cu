@@ -749,7 +749,8 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   int* nSegHits = dalloc<int>(M, nTl + 1);
   int* segPos = dalloc<int>(M, nTl + 1);
   int* segHitPos = dalloc<int>(M, nTl + 1);
-  launch_segments_count(nTl, &C->nTl, secBegin, wide, w, tb, nSeg, nSegHits, st);
+  unsigned* ownBits = dalloc<unsigned>(M, (size_t)nTl * kOwnWords);
+  launch_segments_count(nTl, &C->nTl, secBegin, wide, w, tb, nSeg, nSegHits, ownBits, st);
   CKL();
   scan_exclusive(nSeg, segPos, nTl, &C->nTl, scratch, st);
   CKL();
@@ -774,12 +775,10 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   sb.orig = dalloc<int>(M, nStHits);
   sb.in = dalloc<float>(M, (size_t)nSt * 21);
   sb.out = dalloc<float>(M, (size_t)nSt * 21);
-  launch_segments_write(nTl, &C->nTl, secBegin, wide, w, tb, segPos, segHitPos, syz, sorig, sb, nSt, nStHits, st);
+  launch_segments_write(nTl, &C->nTl, tb, ownBits, segPos, segHitPos, syz, sorig, sb, nSt, nStHits, st);
   CKL();
   // CSR end: sb.off[nSt] = nStHits
   launch_count_at(segPos, &C->nTl, &C->nSt, nSt, &C->overflow, st, segHitPos, &C->nStHits, nStHits, sb.off);
-  CKL();
-  launch_st_gather(nStHits, &C->nStHits, sb, syz, sorig, st);
   CKL();
   CK(cudaEventRecord(c->evs[6], st));
   int* stPerm = dalloc<int>(M, nSt);

@@ -93,6 +93,7 @@ size_t graph_carve(GraphArena& A, char* base) {
   take(A.w, n);
   take(A.secBegin, k.BCap * kNSec + 1);
   take(A.wide, 1);
+  take(A.ownBits, (size_t)k.tlCap * kOwnWords);
   take(A.nSeg, k.tlCap + 1);
   take(A.nSegHits, k.tlCap + 1);
   take(A.segPos, k.tlCap + 1);
@@ -193,14 +194,13 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   // A9
   cudaMemsetAsync(A.w, 0, sizeof(unsigned long long) * (size_t)n, st);
   launch_ownership(k.tlCap, &C->nTl, k.BCap * kNSec, A.grid, A.starts, A.tb, A.w, A.secBegin, A.wide, st);
-  launch_segments_count(k.tlCap, &C->nTl, A.secBegin, A.wide, A.w, A.tb, A.nSeg, A.nSegHits, st);
+  launch_segments_count(k.tlCap, &C->nTl, A.secBegin, A.wide, A.w, A.tb, A.nSeg, A.nSegHits, A.ownBits, st);
   scan_exclusive(A.nSeg, A.segPos, k.tlCap, &C->nTl, A.scratch, st);
   scan_exclusive(A.nSegHits, A.segHitPos, k.tlCap, &C->nTl, A.scratch, st);
-  launch_segments_write(k.tlCap, &C->nTl, A.secBegin, A.wide, A.w, A.tb, A.segPos, A.segHitPos, A.syz, A.sorig,
-                        A.sb, k.stCap, k.stHitsCap, st);
+  launch_segments_write(k.tlCap, &C->nTl, A.tb, A.ownBits, A.segPos, A.segHitPos, A.syz, A.sorig, A.sb, k.stCap,
+                        k.stHitsCap, st);
   launch_count_at(A.segPos, &C->nTl, &C->nSt, k.stCap, &C->overflow, st, A.segHitPos, &C->nStHits, k.stHitsCap,
                   A.sb.off);
-  launch_st_gather(k.stHitsCap, &C->nStHits, A.sb, A.syz, A.sorig, st);
   launch_sector_fit(k.stCap, &C->nSt, A.workCounter + 4, A.perm, A.tb, G, A.sb, st);
   launch_iota(A.tfKeys, k.BCap + 1, st);
   launch_lower_bounds(A.sb.tf, &C->nSt, A.tfKeys, k.BCap + 1, A.stTfBegin, st);

@@ -39,6 +39,7 @@ struct GraphArena {
   int* workCounter;
   int* perm;  // processing order of the passes
   unsigned long long* w;
+  unsigned* ownBits;
   int *secBegin, *wide, *nSeg, *nSegHits, *segPos, *segHitPos;
   SectorTrackBufs sb;
   int *stTfBegin, *tfKeys;

@@ -137,15 +137,15 @@ struct SectorTrackBufs {
 // sector ranges; w must hold 8 bytes per hit and start at zero).
 void launch_ownership(int nTl, const int* nTlDev, int nSec, const RowGrid* grid, const int* starts, TrackletBufs tb,
                       void* w, int* secBegin, int* wide, cudaStream_t st);
+// ownBits: kOwnWords words per tracklet, the ownership of its hits for the
+// write pass.
+constexpr int kOwnWords = (kMaxTlHits + 31) / 32;
 void launch_segments_count(int nTl, const int* nTlDev, const int* secBegin, const int* wide, const void* w,
-                           TrackletBufs tb, int* nSeg, int* nSegHits, cudaStream_t st);
+                           TrackletBufs tb, int* nSeg, int* nSegHits, unsigned* ownBits, cudaStream_t st);
 // capSt / capHits: room in the sector-track buffers (writes past them dropped)
-void launch_segments_write(int nTl, const int* nTlDev, const int* secBegin, const int* wide, const void* w,
-                           TrackletBufs tb, const int* segPos, const int* segHitPos, const int2* syz,
-                           const int* sorig, SectorTrackBufs sb, int capSt, int capHits, cudaStream_t st);
-// sb.yz / sb.orig of every sector-track hit (after the CSR end is written)
-void launch_st_gather(int nHits, const int* nHitsDev, SectorTrackBufs sb, const int2* syz, const int* sorig,
-                      cudaStream_t st);
+void launch_segments_write(int nTl, const int* nTlDev, TrackletBufs tb, const unsigned* ownBits, const int* segPos,
+                           const int* segHitPos, const int2* syz, const int* sorig, SectorTrackBufs sb, int capSt,
+                           int capHits, cudaStream_t st);
 // perm (here, in the tracklet passes and in the final refit): scratch for the
 // processing order, one int per item; counter: a zeroed work counter.
 void launch_sector_fit(int nSt, const int* nStDev, int* counter, int* perm, const TrackletBufs tb, const GeomConst* G,
