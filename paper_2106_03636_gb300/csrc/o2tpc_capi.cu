@@ -701,7 +701,7 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
                     upRaw, dnRaw, dErr, st, c->cfg.debug_inject);
   CKL();
   if (c->cfg.flags & O2TPC_FLAG_ROW_STEP2) {
-    launch_neighbours_gap(n, &C->n, grid, nRows, cellStart, syz, G, upRaw, dnRaw, st);
+    launch_neighbours_gap(nfBlocksMax, nfB, nfBlockStart, grid, nRows, cellStart, syz, G, zv, upRaw, dnRaw, st);
     CKL();
   }
   CK(cudaEventRecord(c->evs[3], st));

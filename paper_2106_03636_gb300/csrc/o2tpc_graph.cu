@@ -183,7 +183,9 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   // A5-A7
   launch_neighbours(n / nfBlock + k.nRows + 1, nfBlock, nfStage, A.grid, A.nfBlockStart, k.nRows, A.cellStart, A.syz, G, zv,
                     A.upRaw, A.dnRaw, A.err, st);
-  if (rowStep2) launch_neighbours_gap(n, &C->n, A.grid, k.nRows, A.cellStart, A.syz, G, A.upRaw, A.dnRaw, st);
+  if (rowStep2)
+    launch_neighbours_gap(n / nfBlock + k.nRows + 1, nfBlock, A.nfBlockStart, A.grid, k.nRows, A.cellStart, A.syz, G, zv,
+                          A.upRaw, A.dnRaw, st);
   launch_clean(n, &C->n, A.upRaw, A.dnRaw, A.up, A.dn, A.flag, st);
   launch_ballot_count(n, &C->n, A.flag, A.tileCnt, A.tileOff, &C->nTl, k.tlCap, &C->overflow, A.scratch, st);
   launch_ballot_compact(n, &C->n, A.flag, A.tileOff, A.starts, k.tlCap, &C->overflow, st);

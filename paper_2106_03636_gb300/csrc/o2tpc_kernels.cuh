@@ -45,9 +45,10 @@ void launch_neighbours(int nfBlocks, int hitsPerBlock, bool stage, const RowGrid
                        int nRows, const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw,
                        int* dnRaw, unsigned* err, cudaStream_t st, unsigned inject = 0);
 // Row step 2: links across one missing row for the hits that found no
-// adjacent-row pair (after launch_neighbours; n sizes the grid).
-void launch_neighbours_gap(int n, const int* nDev, const RowGrid* grid, int nRows, const int* cellStart,
-                           const int2* syz, const GeomConst* G, int* upRaw, int* dnRaw, cudaStream_t st);
+// adjacent-row pair (after launch_neighbours, with the same blocks).
+void launch_neighbours_gap(int nfBlocks, int hitsPerBlock, const int* nfBlockStart, const RowGrid* grid, int nRows,
+                           const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw, int* dnRaw,
+                           cudaStream_t st);
 // Data-dependent sizes are read by the kernels from device memory (nDev,
 // the fields of Counts); the host-side n of a launcher only sizes its grid:
 // the exact size on the regular path, a capacity on the captured path.

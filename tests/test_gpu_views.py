@@ -39,6 +39,21 @@ def test_views_against_the_oracle(kind):
 
 
 @pytest.mark.parametrize("kind", ["dense", "lumps", "sparse", "one_time"])
+def test_row_step2_views_against_the_oracle(kind):
+    """Links across a missing row, bit for bit, with a seventh of the rows' hits gone."""
+    tf = _frame(kind)
+    keep = np.random.default_rng(1).random(tf.n) > 1.0 / 7.0
+    tf.sector, tf.row, tf.y, tf.z = (np.ascontiguousarray(a[keep]) for a in (tf.sector, tf.row, tf.y, tf.z))
+    tf.n = int(keep.sum())
+    with o2tpc.Tracker(flags=o2tpc.O2TPC_FLAG_KEEP_STAGES | o2tpc.O2TPC_FLAG_ROW_STEP2) as t:
+        ticket = t.submit(tf)
+        res = t.poll(ticket, keep=True)
+        assert res["status"] == 0
+        compare_stages(t, ticket, oracle.run(tf, row_step2=True))
+        t.release(ticket, res)
+
+
+@pytest.mark.parametrize("kind", ["dense", "lumps", "sparse", "one_time"])
 def test_cooperative_search_in_the_cells_agrees(kind):
     """The warp-cooperative search looks through the cells: the same tracks."""
     tf = _frame(kind)
