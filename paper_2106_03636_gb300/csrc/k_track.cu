@@ -144,11 +144,18 @@ __global__ void __launch_bounds__(128) k_tl_chain(const int* __restrict__ nTlDev
     H[0] = h0;
     Rw[0] = (uint8_t)r0;
     int nc = 1, hit = h1, prev = r0, Rh = R1;
+    int2 hn = syz[h1];
+    int next = h2;
     bool dropped = false;
     while (hit >= 0 && nc < kMaxTlHits) {
       const int row = r0 + (Rh - R0);
-      const int2 hp = syz[hit];  // both loads in flight during the transport
-      const int next = up[hit];
+      // the next hit's coordinates and link, in flight during this hit's step
+      const int2 hp = hn;
+      int after = -1;
+      if (next >= 0) {
+        hn = syz[next];
+        after = up[next];
+      }
       if (kf_prop_row<float, kF1Rounded>(st, prev, row, G, bzc) != 0) {
         dropped = true;
         break;
@@ -160,6 +167,7 @@ __global__ void __launch_bounds__(128) k_tl_chain(const int* __restrict__ nTlDev
       ++nc;
       prev = row;
       hit = next;
+      next = after;
       if (hit >= 0) Rh = link_row(grid, Rh, hit, rs2);
     }
     tb.nasc[k] = dropped ? 0 : nc;
