@@ -213,7 +213,7 @@ __device__ inline int upper_bound_i32(const int* a, int n, int v) {
 
 // ---------------------------------------------- work in order of length
 // Persistent warps: the next 32 of n items, in the order perm (see
-// launch_length_order); item: this lane's, -1 if there is none for it.  False
+// launch_length_order; null: plain order); item: this lane's, -1 if there is none for it.  False
 // when no items are left.  All lanes call it.
 __device__ inline bool take_ordered(int* counter, const int* __restrict__ perm, int n, int& item) {
   const int lane = threadIdx.x & 31;
@@ -221,7 +221,7 @@ __device__ inline bool take_ordered(int* counter, const int* __restrict__ perm, 
   if (lane == 0) j = atomicAdd(counter, 32);
   j = __shfl_sync(0xffffffffu, j, 0);
   if (j >= n) return false;
-  item = j + lane < n ? perm[j + lane] : -1;
+  item = j + lane < n ? (perm ? perm[j + lane] : j + lane) : -1;
   return true;
 }
 
