@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(kT) k_cell_sort(const RowGrid* __restrict__ gr
 // may be shared with the chunk before, whose hits come first): every chunk is
 // counted, scanned and scattered by itself in shared memory, its output range
 // is its input range, and the writes stay inside it.  Bound by memory: 8
-// bytes read (twice, the second time from L2), 12 + 4 per bin written per hit.
+// bytes read (twice, the second time from L2), 10 + 2 per bin written per hit.
 constexpr int kZBins = 4096, kZThreads = 256;
 // Units, 0.5 cm at 2.58 cm/us: half a following window.  1 cm: following 3 %, the
 // NeighboursFinder 6 % slower on 16 orbits; 2 cm: 18 and 30 %.
@@ -506,8 +506,10 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
   if (threadIdx.x == 0) zrow[blockIdx.x] = z;
   char* mem = reinterpret_cast<char*>(bucket) + 16ll * g.start;
   int2* yz = reinterpret_cast<int2*>(mem);
-  int* idx = reinterpret_cast<int*>(mem + 8ll * g.count);
-  int* bins = reinterpret_cast<int*>(mem + 12ll * g.count);
+  short* idx = reinterpret_cast<short*>(mem + 8ll * g.count);
+  unsigned short* bins16 = reinterpret_cast<unsigned short*>(mem + 12ll * g.count);
+  int* bins32 = reinterpret_cast<int*>(mem + 12ll * g.count);
+  bool far = false;  // an index distance beyond 16 bits
   const float perCellRow = (float)g.cz * z.zinv * 1.0001f + 1.f;
   const int izPer = max(1, (int)((float)(kZBins - 8) / perCellRow));
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -544,7 +546,10 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
     for (int c = c0; c < c1; ++c) {
       const int v = s_cnt[c];
       s_cnt[c] = off;
-      if (c > 0) bins[bL + c] = base + off;
+      if (c > 0) {
+        if (g.count <= kZShortRow) bins16[bL + c] = (unsigned short)(base + off);
+        else bins32[bL + c] = base + off;
+      }
       off += v;
     }
     __syncthreads();
@@ -553,11 +558,15 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
       const int b = z_bin(p.y, g.zmin, z.zinv, z.nzb);
       const int pos = base + atomicAdd(&s_cnt[min(max(b - bL, 0), nb)], 1);
       yz[pos] = p;
-      idx[pos] = h;
+      const int d = h - g.start - pos;
+      idx[pos] = (short)d;
+      far = far || d != (int)(short)d;
     }
     __syncthreads();
     bL = bR;
   }
+  // too far apart: the searches of this row's neighbourhood take the cells
+  if (__syncthreads_or(far) && threadIdx.x == 0) zrow[blockIdx.x].flags = kZNFCells | kZFollowCells;
 }
 
 // ------------------------------------------------------------- launchers

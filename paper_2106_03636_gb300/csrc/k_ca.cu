@@ -131,8 +131,6 @@ __device__ inline void nf_view(const ZView& V, const ZRow& gu, const ZRow& gd, i
                                int& bu, int& bd) {
   const int2* pu = V.yz(gu);
   const int2* pd = V.yz(gd);
-  const int* iu = V.idx(gu);
-  const int* id = V.idx(gd);
   auto inside = [&](int2 c) {
     return (unsigned)(hh.x - c.x + kWinY) <= 2u * kWinY && (unsigned)(hh.y - c.y + kWinZ) <= 2u * kWinZ;
   };
@@ -144,8 +142,8 @@ __device__ inline void nf_view(const ZView& V, const ZRow& gu, const ZRow& gd, i
   auto take = [&](int D, int u, int d) {
     bool better = D < bestD;
     if (D == bestD && pbu >= 0) {
-      const int a = __ldg(iu + u), b = __ldg(iu + pbu);
-      better = a < b || (a == b && __ldg(id + d) < __ldg(id + pbd));
+      const int a = V.idx(gu, u), b = V.idx(gu, pbu);
+      better = a < b || (a == b && V.idx(gd, d) < V.idx(gd, pbd));
     }
     if (better) {
       bestD = D;
@@ -242,8 +240,8 @@ __device__ inline void nf_view(const ZView& V, const ZRow& gu, const ZRow& gd, i
     }
   }
   if (pbu >= 0) {
-    bu = __ldg(iu + pbu);
-    bd = __ldg(id + pbd);
+    bu = V.idx(gu, pbu);
+    bd = V.idx(gd, pbd);
   }
 }
 
@@ -292,7 +290,7 @@ __global__ void __launch_bounds__(kB) k_neighbours_view(const RowGrid* __restric
     return;
   }
   const int2 hh = zv.yz(g)[q];
-  const int h = zv.idx(g)[q];
+  const int h = zv.idx(g, q);
   const ZRow gu = zv.rows[R + 1], gd = zv.rows[R - 1];
   int bu = -1, bd = -1;
   if ((gu.flags | gd.flags) & kZNFCells) {
@@ -509,7 +507,6 @@ __device__ inline void gap_view(const ZView& V, const ZRow& gu, const ZRow& gd, 
   if (!z_range(V, gu, hh.y - a * kWinZ, hh.y + a * kWinZ, ua, ub)) return;
   if (!z_range(V, gd, hh.y - b * kWinZ, hh.y + b * kWinZ, da, db)) return;
   const int2 *pu = V.yz(gu), *pd = V.yz(gd);
-  const int *iu = V.idx(gu), *id = V.idx(gd);
   const int f = (a + b) * (a + b) + a * a + b * b;
   auto inside = [&](int2 c, int w) {
     return (unsigned)(hh.x - c.x + w * kWinY) <= 2u * w * kWinY && (unsigned)(hh.y - c.y + w * kWinZ) <= 2u * w * kWinZ;
@@ -536,7 +533,7 @@ __device__ inline void gap_view(const ZView& V, const ZRow& gu, const ZRow& gd, 
           // past the cut for every f (<= 24): 6 * 2077 * 320^2 and 6 * 1536 * 370^2 > kMaxMetric * 24
           if (abs(ey) > 320 || abs(ez) > 370) continue;
           const long long D = (long long)(kWeightY * ey * ey) + (long long)(kWeightZ * ez * ez);
-          if (6 * D <= (long long)kMaxMetric * f) best.offer(D, f, __ldg(iu + u), __ldg(id + d));
+          if (6 * D <= (long long)kMaxMetric * f) best.offer(D, f, V.idx(gu, u), V.idx(gd, d));
         }
       }
     }
@@ -561,7 +558,7 @@ __global__ void __launch_bounds__(kB) k_neighbours_gap(const int* __restrict__ n
   const ZRow g = zv.rows[R];
   const int q = (blockIdx.x - nfBlockStart[R]) * kB + threadIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const bool free = q < g.count && upRaw[zv.idx(g)[q]] < 0;
+  const bool free = q < g.count && upRaw[zv.idx(g, q)] < 0;
   const unsigned m = __ballot_sync(0xffffffffu, free);
   if (lane == 0) s_cnt[w] = __popc(m);
   __syncthreads();
@@ -588,7 +585,7 @@ __global__ void __launch_bounds__(kB) k_neighbours_gap(const int* __restrict__ n
       gap_view(zv, gu, gd, a, b, hh, best);
   }
   if (best.u >= 0) {
-    const int h = zv.idx(g)[p];
+    const int h = zv.idx(g, p);
     upRaw[h] = best.u;
     dnRaw[h] = best.d;
   }

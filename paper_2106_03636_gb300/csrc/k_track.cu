@@ -322,8 +322,8 @@ __device__ inline unsigned long long cand_key(int h, int2 p, const SearchPar& P,
   return ((unsigned long long)__float_as_uint(chi) << 32) | (unsigned)h;
 }
 
-// Best hit of a search: its index in the list `idx` of sorted indices (null:
-// it is the sorted index itself; -1: none) and its coordinates.
+// Best hit of a search: its place in the row's view (cells: its sorted index),
+// -1 for none, and its coordinates.
 struct BestHit {
   int pos;
   int2 p;
@@ -357,8 +357,8 @@ __device__ inline BestHit cell_search(const RowGrid& g, int iy0, int iy1, int iz
 // four candidates loaded at once (a window holds 3-4 on average), so a row
 // step waits for one load and not for one per candidate.  Equal chi2 (rare)
 // goes to the smaller sorted index.
-__device__ inline BestHit z_search(const int2* __restrict__ yz, const int* __restrict__ idx, int a, int b,
-                                   const SearchPar& P, float zunit) {
+__device__ inline BestHit z_search(const ZView& V, const ZRow& g, int a, int b, const SearchPar& P, float zunit) {
+  const int2* yz = V.yz(g);
   unsigned best = ~0u;
   bool tie = false;
   BestHit B{-1, make_int2(0, 0)};
@@ -385,7 +385,7 @@ __device__ inline BestHit z_search(const int2* __restrict__ yz, const int* __res
   if (tie) {
     for (int h = a; h < b; ++h) {
       const int2 q = __ldg(yz + h);
-      if ((unsigned)(cand_key(0, q, P, zunit) >> 32) == best && __ldg(idx + h) < __ldg(idx + B.pos)) {
+      if ((unsigned)(cand_key(0, q, P, zunit) >> 32) == best && V.idx(g, h) < V.idx(g, B.pos)) {
         B.pos = h;
         B.p = q;
       }
@@ -594,9 +594,9 @@ __global__ void __launch_bounds__(128, 7) k_tl_follow_coop(const int* __restrict
 // direction parameters and the row of the last accepted state (with kKeep the
 // whole state, for inspection), so nothing is copied per accepted hit.
 // Measured against the search in the cells with the state copied per hit:
-// 1 ms frame (20.3 M clusters) 2.26 + 1.73 -> 1.59 + 1.31 ms, 32 orbits (59 M)
-// 6.87 + 5.19 -> 4.73 + 3.97 ms, 3 collisions (1.3 M, one tracklet a lane)
-// 0.58 + 0.55 -> 0.37 + 0.45 ms.
+// 1 ms frame (20.3 M clusters) 2.26 + 1.73 -> 1.51 + 1.26 ms, 32 orbits (59 M)
+// 6.87 + 5.19 -> 4.45 + 3.75 ms, 3 collisions (1.3 M, one tracklet a lane)
+// 0.58 + 0.55 -> 0.38 + 0.44 ms.
 // The list index of the hit is loaded off the step's chain (beside the
 // update).  Loading the next row's bin starts ahead (prefetch to L1 or L2) cost
 // 6 %.  Blocks of 128 per SM the kernel is compiled for: 7 (72 registers)
@@ -604,6 +604,11 @@ __global__ void __launch_bounds__(128, 7) k_tl_follow_coop(const int* __restrict
 #ifndef O2TPC_FOLLOW_MIN_BLOCKS
 #define O2TPC_FOLLOW_MIN_BLOCKS 7
 #endif
+
+// Tracklets a warp reserves at a time: 1 (an atomic for every refill) measured 1.54 +
+// 1.27 ms on the 1 ms frame, 8 1.51 + 1.26, 32 1.67 + 1.46 (the tracklets in
+// flight, and what they touch, spread out: L2 hits 47 -> 38 %).
+constexpr int kFollowBatch = 8;
 
 template <int kDir, bool kKeep>
 __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
@@ -616,6 +621,8 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
   const float zunit = G->zunit, izunit = G->kz, bzc = G->bzc;
   const int angErr = G->angErr;
   const int nTl = *nTlDev;
+  const int lane = threadIdx.x & 31;
+  int batch = 0, batchEnd = 0;
   bool have = false, exhausted = false;
   int k = 0, r = 0, n = 0, misses = 0, srow = 0, yref = 0, yrefLast = 0, zref = 0, Rs = 0, lastRow = 0;
   float last2 = 0.f, last3 = 0.f, last4 = 0.f;
@@ -655,27 +662,43 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
     have = false;
   };
   for (;;) {
-    // lanes without a tracklet take the next ones
+    // lanes without a tracklet take the next ones (the warp reserves a few at a
+    // time); their loads depend on the index alone
     const bool want = !have && !exhausted;
-    const int kk = warp_take(counter, want);
-    if (want) {
-      k = kk;
-      if (k >= nTl) {
-        exhausted = true;
-      } else {
-        const int na = tb.nasc[k];
-        if (na > 0) {
-          const uint8_t* Rw = tb.rows + (size_t)k * kMaxTlHits;
+    const unsigned wants = __ballot_sync(full, want);
+    if (wants) {
+      const int cnt = __popc(wants), rank = __popc(wants & ((1u << lane) - 1u)), left = batchEnd - batch;
+      int kk = batch + rank;
+      batch += cnt;
+      if (cnt > left) {
+        const int take = max(cnt - left, kFollowBatch);
+        int nb = 0;
+        if (lane == 0) nb = atomicAdd(counter, take);
+        nb = __shfl_sync(full, nb, 0);
+        if (rank >= left) kk = nb + rank - left;
+        batch = nb + cnt - left;
+        batchEnd = nb + take;
+      }
+      if (want) {
+        k = kk;
+        if (k >= nTl) {
+          exhausted = true;
+        } else {
+          const int na = tb.nasc[k];
+          const int row0 = tb.rows[(size_t)k * kMaxTlHits];
           Rs = tb.rbase[k];
           zref = tb.zref[k];
           yref = tb.yref[k];
           load_state(st, tb.state + (size_t)k * 21);
-          n = na;
-          r = (kDir > 0) ? Rw[na - 1] + 1 : Rw[0] - 1;
-          misses = 0;
-          srow = row_of_x(st.x);
-          save_last();
-          have = true;
+          if (na > 0) {
+            n = na;
+            misses = 0;
+            srow = row_of_x(st.x);
+            // the chain's last fitted hit is its top; the refit may have skipped the lowest
+            r = (kDir > 0) ? srow + 1 : row0 - 1;
+            save_last();
+            have = true;
+          }
         }
       }
     }
@@ -685,7 +708,7 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
     }
     // one row step of every busy lane: transport, then the window
     BestHit best{-1, make_int2(0, 0)};
-    const int* idx = nullptr;
+    ZRow gv{};  // the row of best.pos; count 0: best.pos is the sorted index
     if (have) {
       if ((kDir > 0) ? (r >= kNRow) : (r < 0)) {
         finish();
@@ -706,8 +729,9 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
           } else {
             int a, b;
             if (z_range(zv, g, zlo, zhi, a, b)) {
-              idx = zv.idx(g);
-              best = z_search(zv.yz(g), idx, a, b, P, zunit);
+              best = z_search(zv, g, a, b, P, zunit);
+              gv.start = g.start;
+              gv.count = g.count;
             }
           }
         }
@@ -715,7 +739,7 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
     }
     if (have) {
       if (best.pos >= 0) {
-        const int hit = idx ? __ldg(idx + best.pos) : best.pos;  // in flight during the update
+        const int hit = gv.count ? zv.idx(gv, best.pos) : best.pos;  // in flight during the update
         recentre_y(st.p[0], yref, best.p.x);
         kf_update<float>(st, hit_y(best.p.x, yref), hit_z(best.p.y, zref, zunit), nullptr, angErr);
         tb.rows[(size_t)k * kMaxTlHits + n] = (uint8_t)r;

@@ -79,8 +79,10 @@ struct RowGrid {
 // holds 2-8 hits of a whole pad row at 50 kHz Pb-Pb, where the cells of the
 // sorted order (2 cm x 40-110 cm there: 4 hits each) that cover the same
 // window hold 10 or more.  The view lives in the row's bucket records, which
-// the cell sort has used up (16 bytes per hit: coordinates 8, sorted index 4,
-// bin starts 4 - so a row has at most as many bins as hits).
+// the cell sort has used up: coordinates (8 bytes a hit), the sorted index as a
+// 16-bit distance from the place (the two orders differ inside a cell row), bin
+// starts (16 bits; 32 in rows of more hits - a row has at most as many bins as
+// hits).  What a batch's concurrent searches touch has to stay in L2.
 struct ZRow {
   int start;    // first sorted hit of the row (batch-global), as RowGrid
   int count;
@@ -91,19 +93,32 @@ struct ZRow {
   int pad0, pad1;
 };
 // Rows so dense that the cells hold fewer candidates than the drift window:
-// bit 0 for the NeighboursFinder's window, bit 1 for the following's.
+// bit 0 for the NeighboursFinder's window, bit 1 for the following's.  Both are
+// set when the orders lie too far apart for the 16-bit distances.
 enum : int { kZNFCells = 1, kZFollowCells = 2 };
+constexpr int kZShortRow = 65535;  // hits of a row with 16-bit bin starts, at most
 
 // The drift-ordered views of a batch: row tables and the record memory.
 struct ZView {
   const ZRow* rows;
   const char* mem;
   __device__ const int2* yz(const ZRow& g) const { return reinterpret_cast<const int2*>(mem + 16ll * g.start); }
-  __device__ const int* idx(const ZRow& g) const {
-    return reinterpret_cast<const int*>(mem + 16ll * g.start + 8ll * g.count);
+  // sorted index of the hit at a place
+  __device__ int idx(const ZRow& g, int place) const {
+    return g.start + place + (int)__ldg(reinterpret_cast<const short*>(mem + 16ll * g.start + 8ll * g.count) + place);
   }
-  __device__ const int* bins(const ZRow& g) const {
-    return reinterpret_cast<const int*>(mem + 16ll * g.start + 12ll * g.count);
+  // first places of bins b0 and b1 (b1 may be nzb: the row's end)
+  __device__ void bins(const ZRow& g, int b0, int b1, int& a, int& b) const {
+    const char* p = mem + 16ll * g.start + 12ll * g.count;
+    const int bl = b1 < g.nzb ? b1 : b0;  // both loads at once
+    if (g.count <= kZShortRow) {
+      a = (int)__ldg(reinterpret_cast<const unsigned short*>(p) + b0);
+      b = (int)__ldg(reinterpret_cast<const unsigned short*>(p) + bl);
+    } else {
+      a = __ldg(reinterpret_cast<const int*>(p) + b0);
+      b = __ldg(reinterpret_cast<const int*>(p) + bl);
+    }
+    if (b1 >= g.nzb) b = g.count;
   }
 };
 
@@ -121,9 +136,7 @@ __device__ inline bool z_range(const ZView& V, const ZRow& g, int zlo, int zhi, 
   if (g.count == 0 || zhi < g.zmin) return false;
   const int b0 = zlo <= g.zmin ? 0 : z_bin(zlo, g.zmin, g.zinv, g.nzb);
   const int b1 = z_bin(zhi, g.zmin, g.zinv, g.nzb);
-  const int* zs = V.bins(g);
-  a = __ldg(zs + b0);
-  b = b1 + 1 < g.nzb ? __ldg(zs + b1 + 1) : g.count;
+  V.bins(g, b0, b1 + 1, a, b);
   return a < b;
 }
 
