@@ -292,7 +292,7 @@ __device__ inline int stream_of_chunk(const CtfStream* __restrict__ sd, int nSd,
 // One block per kCtfHistChunks consecutive chunks (mostly one stream): a
 // shared-memory histogram, flushed to the stream's global one whenever the
 // stream changes.
-constexpr int kCtfHistChunks = 32;
+constexpr int kCtfHistChunks = 8;
 __global__ void __launch_bounds__(256) k_ctf_hist(const int* __restrict__ nChunksDev, const CtfStream* __restrict__ sd,
                                                   int nSd, const uint8_t* __restrict__ sym,
                                                   unsigned* __restrict__ hist) {
@@ -314,14 +314,24 @@ __global__ void __launch_bounds__(256) k_ctf_hist(const int* __restrict__ nChunk
     // runs of equal symbols seen by a thread are added at once (most byte
     // planes are dominated by one symbol)
     unsigned cur = 256u, run = 0;
-    for (long long i = a + threadIdx.x; i < e; i += blockDim.x) {
-      const unsigned v = p[i];
-      if (v == cur) {
-        ++run;
-      } else {
-        if (run) atomicAdd(&h[cur], run);
-        cur = v;
-        run = 1;
+    constexpr int kU = 8;  // symbols in flight per thread
+    for (long long i0 = a + threadIdx.x; i0 < e; i0 += kU * blockDim.x) {
+      unsigned v[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const long long i = i0 + u * (long long)blockDim.x;
+        v[u] = i < e ? p[i] : 256u;
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        if (v[u] == 256u) continue;
+        if (v[u] == cur) {
+          ++run;
+        } else {
+          if (run) atomicAdd(&h[cur], run);
+          cur = v[u];
+          run = 1;
+        }
       }
     }
     if (run) atomicAdd(&h[cur], run);
@@ -335,49 +345,83 @@ __global__ void __launch_bounds__(256) k_ctf_hist(const int* __restrict__ nChunk
   }
 }
 
-// One thread per (TF, stream): the normalised table and its cumulative sums.
-__global__ void k_ctf_norm(int nSd, const unsigned* __restrict__ hist, uint16_t* __restrict__ freq,
-                           uint2* __restrict__ enc, int* __restrict__ degen) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nSd) return;
-  const unsigned* c = hist + s * 256;
-  uint16_t* f = freq + s * 256;
+// Coding entry of a symbol with cumulative start c and frequency f: what the
+// state update x -> (x / f) 4096 + x mod f + c = x + c + (x / f) (4096 - f)
+// needs.  x / f by a multiplication with a rounded-up reciprocal (Granlund and
+// Montgomery 1994, Thm. 4.2): with s = ceil(log2 f) and
+// r = ceil(2^(31 + s) / f), floor(x r / 2^(31 + s)) = floor(x / f) for every
+// x < 2^31, and states stay below 2^31.  r < 2^32 for f >= 2; f = 1 takes
+// r = 2^32 - 1 and no shift, which gives x - 1 for x >= 1, and the missing
+// 4095 goes into the constant.  .x: r; .y: constant | (4096 - f) << 13 | shift << 26.
+__device__ inline uint2 ctf_entry(unsigned c, unsigned f) {
+  if (f == 0) return make_uint2(0u, 0u);
+  if (f == 1) return make_uint2(~0u, (c + kCtfM - 1u) | ((kCtfM - 1u) << 13));
+  const unsigned s = 32u - (unsigned)__clz(f - 1u);  // ceil(log2 f)
+  const unsigned r = (unsigned)(((1ull << (31 + s)) + f - 1u) / f);
+  return make_uint2(r, c | ((kCtfM - f) << 13) | ((s - 1u) << 26));
+}
+
+// One warp per (TF, stream), eight consecutive symbols a lane: the normalised
+// table and its cumulative sums.  (A thread walking all 256 symbols several
+// times took 96 us.)
+__global__ void __launch_bounds__(32) k_ctf_norm(const unsigned* __restrict__ hist, uint16_t* __restrict__ freq,
+                                                 uint2* __restrict__ enc, int* __restrict__ degen) {
+  const unsigned full = 0xffffffffu;
+  const int s = blockIdx.x, lane = threadIdx.x;
+  unsigned c[8], f[8];
   unsigned long long n = 0;
-  for (int k = 0; k < 256; ++k) n += c[k];
-  long long sum = 0;
-  for (int k = 0; k < 256; ++k) {
-    unsigned long long v = 0;
-    if (c[k]) {
-      v = (unsigned long long)c[k] * kCtfM / n;
-      if (v < 1) v = 1;
-    }
-    f[k] = (uint16_t)v;
-    sum += (long long)v;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    c[k] = hist[s * 256 + lane * 8 + k];
+    n += c[k];
   }
-  long long dlt = n ? (long long)kCtfM - sum : 0;
-  while (dlt != 0) {
-    int best = -1;
-    for (int k = 0; k < 256; ++k)
-      if (f[k] && (best < 0 || f[k] > f[best])) best = k;
-    if (dlt > 0) {
-      f[best] = (uint16_t)(f[best] + dlt);
-      dlt = 0;
-    } else {
-      long long take = (long long)f[best] - 1;
-      if (take > -dlt) take = -dlt;
-      f[best] = (uint16_t)(f[best] - take);
-      dlt += take;
-    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(full, n, o);
+  int sum = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    f[k] = c[k] ? max((unsigned)((unsigned long long)c[k] * kCtfM / n), 1u) : 0u;
+    sum += (int)f[k];
   }
-  // coding entries: cumulative start | frequency << 16, and 1 / frequency
-  unsigned acc = 0;
-  int dg = 0;
-  for (int k = 0; k < 256; ++k) {
-    enc[s * 256 + k] = make_uint2(acc | ((unsigned)f[k] << 16), __float_as_uint(f[k] ? 1.0f / (float)f[k] : 0.f));
+  sum = __reduce_add_sync(full, sum);
+  int dlt = n ? (int)kCtfM - sum : 0;
+  while (dlt != 0) {  // to the largest entry, the lower symbol first
+    unsigned key = 0;  // frequency << 8 | 255 - symbol of the lane's best (0: none)
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (f[k]) key = max(key, (f[k] << 8) | (unsigned)(255 - (lane * 8 + k)));
+    key = __reduce_max_sync(full, key);
+    const int best = 255 - (int)(key & 255u), fb = (int)(key >> 8);
+    const int add = dlt > 0 ? dlt : -min(fb - 1, -dlt);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (lane * 8 + k == best) f[k] = (unsigned)(fb + add);
+    dlt -= add;
+  }
+  // coding entries (ctf_entry)
+  unsigned own = 0;
+  bool dg = false;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    own += f[k];
+    dg |= f[k] == (unsigned)kCtfM;
+  }
+  unsigned acc = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(full, acc, o);
+    if (lane >= o) acc += y;
+  }
+  acc -= own;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = s * 256 + lane * 8 + k;
+    freq[i] = (uint16_t)f[k];
+    enc[i] = ctf_entry(acc, f[k]);
     acc += f[k];
-    dg |= f[k] == kCtfM;
   }
-  degen[s] = dg;
+  dg = __any_sync(full, dg);
+  if (lane == 0) degen[s] = dg;
 }
 
 // One thread per chunk: rANS from the last symbol to the first; the emitted
@@ -385,12 +429,28 @@ __global__ void k_ctf_norm(int nSd, const unsigned* __restrict__ hist, uint16_t*
 // 32-bit words), the final state in front of them.  bytes[c] = 4 + emitted.
 // A table with one symbol of frequency 4096 codes nothing: the state stays
 // at its initial value.
-__global__ void __launch_bounds__(128) k_ctf_encode(const int* __restrict__ nChunksDev, const CtfStream* __restrict__ sd,
-                                                    int nSd, const uint8_t* __restrict__ sym,
-                                                    const uint2* __restrict__ enc, const int* __restrict__ degen,
-                                                    uint8_t* __restrict__ scratch, int* __restrict__ bytes) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= *nChunksDev) return;
+// A chunk is a chain of 4096 states, and there are fewer chunks than GPU
+// threads: the time is the chain's.  The 32 chunks of a block (one warp) are of
+// one stream or two, whose tables lie in shared memory; symbols come four to a
+// load, entries are looked up ahead of the state, the division is a
+// multiplication.  5.4 M clusters: 0.99 ms (two dependent loads, a division and
+// a branch per byte in every step) -> 0.36.
+constexpr int kEncThreads = 32;
+__global__ void __launch_bounds__(kEncThreads) k_ctf_encode(const int* __restrict__ nChunksDev,
+                                                            const CtfStream* __restrict__ sd, int nSd,
+                                                            const uint8_t* __restrict__ sym,
+                                                            const uint2* __restrict__ enc,
+                                                            const int* __restrict__ degen,
+                                                            uint8_t* __restrict__ scratch, int* __restrict__ bytes) {
+  __shared__ uint2 s_tab[2][256];
+  const int nCh = *nChunksDev, c0 = blockIdx.x * kEncThreads;
+  if (c0 >= nCh) return;
+  const int first = stream_of_chunk(sd, nSd, c0);
+  for (int i = threadIdx.x; i < 512; i += kEncThreads)
+    if (first * 256 + i < nSd * 256) s_tab[i >> 8][i & 255] = enc[first * 256 + i];
+  __syncthreads();
+  const int c = c0 + threadIdx.x;
+  if (c >= nCh) return;
   const int s = stream_of_chunk(sd, nSd, c);
   const CtfStream d = sd[s];
   const long long a = (long long)(c - d.chunk0) * kCtfChunk;
@@ -400,35 +460,62 @@ __global__ void __launch_bounds__(128) k_ctf_encode(const int* __restrict__ nChu
   int q = kCtfChunkBytes;  // emitted bytes fill [q, kCtfChunkBytes)
   if (!degen[s]) {
     const uint8_t* p = sym + d.start + a;
-    const uint2* tab = enc + s * 256;
-    unsigned w = 0;  // bytes not yet stored, the latest emitted in the low byte
-    int nw = 0;
-    for (int i = n - 1; i >= 0; --i) {
-      const uint2 e = tab[p[i]];
-      const unsigned fs = e.x >> 16, cs = e.x & 0xffffu;
-      const unsigned xmax = ((kCtfL >> kCtfScaleBits) << 8) * fs;
-      while (x >= xmax) {
-        w = (w << 8) | (x & 0xffu);
-        x >>= 8;
-        if (++nw == 4) {
+    // past the second stream (chunks of a few clusters): the global table
+    const uint2* tab = s - first < 2 ? s_tab[s - first] : enc + s * 256;
+    unsigned long long w = 0;  // bytes not yet stored, the latest emitted in the low byte
+    int nw = 0;                // 0..3 of them between symbols
+    // the table entries of 8 symbols are loaded ahead of their steps: they do
+    // not depend on the state, so a symbol costs the state's arithmetic alone
+    constexpr int kU = 8;
+    uint2 ahead[kU];
+    // symbols i0, i0 - 1, ...: the aligned words around the last of them,
+    // shifted together (kept inside the chunk's own bytes at its start)
+    const unsigned mis = (unsigned)(reinterpret_cast<uintptr_t>(p) & 3u);
+    auto word_at = [&](int i) {  // bytes i .. i + 3 of the chunk, i + mis a multiple of 4 or not
+      const int b0 = (i + (int)mis) & ~3;  // from the aligned base p - mis
+      const unsigned* wp = reinterpret_cast<const unsigned*>(p - mis);
+      const unsigned lo = wp[b0 >> 2], hi = wp[(b0 >> 2) + 1];
+      return __funnelshift_r(lo, hi, 8 * ((i + (int)mis) & 3));
+    };
+    auto fetch = [&](int i0) {
+      unsigned sy[kU];
+      if (i0 >= kU - 1) {
+        const unsigned wl = word_at(i0 - 7), wh = word_at(i0 - 3);
+#pragma unroll
+        for (int u = 0; u < kU; ++u) sy[u] = ((u < 4 ? wh : wl) >> (8 * (3 - (u & 3)))) & 255u;
+      } else {
+#pragma unroll
+        for (int u = 0; u < kU; ++u) sy[u] = p[max(i0 - u, 0)];
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) ahead[u] = tab[sy[u]];
+    };
+    fetch(n - 1);
+    for (int i0 = n - 1; i0 >= 0; i0 -= kU) {
+      uint2 now[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) now[u] = ahead[u];
+      if (i0 >= kU) fetch(i0 - kU);
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        if (i0 - u < 0) break;
+        const uint2 e = now[u];
+        const unsigned comp = (e.y >> 13) & 0x1fffu;  // 4096 - f
+        const unsigned xmax = ((kCtfL >> kCtfScaleBits) << 8) * (kCtfM - comp);
+        // renormalisation: none, one or two bytes (x < 2^31, xmax >= 2^19)
+        const bool one = x >= xmax, two = (x >> 8) >= xmax;
+        const unsigned xr = two ? __byte_perm(x, 0, 0x4401) : (x & 0xffu);  // the bytes, first emitted on top
+        const int nb = (int)one + (int)two;
+        w = (w << (8 * nb)) | (one ? xr : 0u);
+        x >>= 8 * nb;
+        nw += nb;
+        if (nw >= 4) {
+          nw -= 4;
           q -= 4;
-          *reinterpret_cast<unsigned*>(out + q) = w;
-          nw = 0;
+          *reinterpret_cast<unsigned*>(out + q) = (unsigned)(w >> (8 * nw));
         }
+        x = x + (e.y & 0x1fffu) + (__umulhi(x, e.x) >> (e.y >> 26)) * comp;
       }
-      // x / fs: here x < 2^19 fs, so the quotient is below 2^19 and the
-      // single-precision estimate (relative error < 2^-22) is off by at most
-      // one, which one remainder test corrects
-      unsigned qt = __float2uint_rz(__uint2float_rn(x) * __uint_as_float(e.y));
-      int r = (int)(x - qt * fs);
-      if (r < 0) {
-        --qt;
-        r += (int)fs;
-      } else if (r >= (int)fs) {
-        ++qt;
-        r -= (int)fs;
-      }
-      x = (qt << kCtfScaleBits) + (unsigned)r + cs;
     }
     for (int k = 0; k < nw; ++k) out[--q] = (uint8_t)(w >> (8 * (nw - 1 - k)));
   }
@@ -582,8 +669,8 @@ void launch_ctf_symbols(int n, const int* nDev, int nTrk, const int* nTrkDev, in
   cudaMemsetAsync(cb.hist, 0, sizeof(unsigned) * 256 * nSd, st);
   k_ctf_hist<<<(cb.chunkCap + kCtfHistChunks - 1) / kCtfHistChunks, 256, 0, st>>>(cb.counts + 2, cb.sd, nSd, cb.sym,
                                                                                   cb.hist);
-  k_ctf_norm<<<(nSd + 63) / 64, 64, 0, st>>>(nSd, cb.hist, cb.freq, cb.enc, cb.degen);
-  k_ctf_encode<<<(cb.chunkCap + 127) / 128, 128, 0, st>>>(cb.counts + 2, cb.sd, nSd, cb.sym, cb.enc, cb.degen,
+  k_ctf_norm<<<nSd, 32, 0, st>>>(cb.hist, cb.freq, cb.enc, cb.degen);
+  k_ctf_encode<<<(cb.chunkCap + kEncThreads - 1) / kEncThreads, kEncThreads, 0, st>>>(cb.counts + 2, cb.sd, nSd, cb.sym, cb.enc, cb.degen,
                                                           cb.scratch, cb.bytes);
   g_launch_count += 3;
   scan_exclusive(cb.bytes, cb.payOff, cb.chunkCap, cb.counts + 2, scratch, st);
