@@ -360,9 +360,9 @@ void autotune(Ctx* c, int n, int nRows, const int* rowCnt, const int* rowMin, co
   int* up = static_cast<int*>(c->dev_alloc(sizeof(int) * (size_t)n * 2));
   for (int i = 0; i < 3; ++i) {
     CK(cudaEventRecord(es[i][0], st));
-    launch_cell_sort(nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, kSort[i]);
+    launch_cell_sort(n, nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, kSort[i]);
     CK(cudaEventRecord(es[i][1], st));
-    launch_cell_sort(nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, kSort[i]);
+    launch_cell_sort(n, nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, kSort[i]);
     CK(cudaEventRecord(es[i][2], st));
   }
   // the views take the place of the bucket records: after the last cell sort
@@ -677,7 +677,7 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   int* sorig = dalloc<int>(M, n);
   launch_row_scatter(dTF, dTiles, nTiles, tileSize, G, tileStats, grid, bucket, st);
   CKL();
-  launch_cell_sort(nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, c->tune.sort_threads_per_row);
+  launch_cell_sort(n, nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, c->tune.sort_threads_per_row);
   ZRow* zrow = dalloc<ZRow>(M, nRows);
   if ((c->cfg.flags & O2TPC_FLAG_AUTOTUNE) && !c->tune.tuned && n >= (1 << 20))
     autotune(c, n, nRows, rowCnt, rowMin, rowMax, grid, nfBlockStart, totals, bucket, cellStart, syz, sorig, gscratch,

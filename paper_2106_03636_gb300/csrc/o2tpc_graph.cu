@@ -177,7 +177,7 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   launch_row_reduce(A.tfs, k.BCap, A.tileStats, A.rowCnt, A.rowMin, A.rowMax, st);
   launch_grid(k.nRows, A.rowCnt, A.rowMin, A.rowMax, G, A.grid, A.nfBlockStart, nfBlock, A.totals, st);
   launch_row_scatter(A.tfs, A.tiles, k.nTilesCap, k.tileSize, G, A.tileStats, A.grid, A.bucket, st);
-  launch_cell_sort(k.nRows, A.grid, A.bucket, A.cellStart, A.syz, A.sorig, A.gscratch, A.totals, st, sortThreads);
+  launch_cell_sort(n, k.nRows, A.grid, A.bucket, A.cellStart, A.syz, A.sorig, A.gscratch, A.totals, st, sortThreads);
   launch_zorder(k.nRows, A.grid, A.rowMax, A.cellStart, A.syz, A.zrow, A.bucket, st);
   const ZView zv{A.zrow, reinterpret_cast<const char*>(A.bucket)};
   // A5-A7
