@@ -162,11 +162,13 @@ __global__ void __launch_bounds__(512) k_merge_list_sort(MergeBufs mb, int2* __r
 }
 
 // Cholesky chi2 = d^T M^-1 d of a symmetric 5x5 (lower triangle); false if
-// M is not positive definite.
-__device__ inline bool chi2_5(const float* d, const float* M, float& out) {
-  float L[15];
+// M is not positive definite or chi2 exceeds cut.  chi2 is a sum of squares taken
+// row by row of the factor, so a row past the cut decides: most pairs that
+// are no match end at the first or second.
+__device__ inline bool chi2_5(const float* d, const float* M, float cut, float& out) {
+  float L[15], v[5], c = 0.f;
 #pragma unroll
-  for (int i = 0; i < 5; ++i)
+  for (int i = 0; i < 5; ++i) {
 #pragma unroll
     for (int j = 0; j <= i; ++j) {
       float s = M[ix(i, j)];
@@ -179,14 +181,12 @@ __device__ inline bool chi2_5(const float* d, const float* M, float& out) {
         L[ix(i, j)] = s / L[ix(j, j)];
       }
     }
-  float v[5], c = 0.f;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
     float s = d[i];
 #pragma unroll
     for (int k = 0; k < i; ++k) s -= L[ix(i, k)] * v[k];
     v[i] = s / L[ix(i, i)];
     c += v[i] * v[i];
+    if (!(c <= cut)) return false;
   }
   out = c;
   return true;
@@ -254,8 +254,7 @@ __global__ void __launch_bounds__(128) k_merge_pairs(SectorTrackBufs sb, const G
 #pragma unroll
     for (int k = 0; k < 15; ++k) cs[k] = t.C[k] + B[6 + k];
     float c2;
-    if (!chi2_5(dv, cs, c2)) continue;
-    if (!(c2 <= kChi2Merge)) continue;
+    if (!chi2_5(dv, cs, kChi2Merge, c2)) continue;
     const int slot = atomicAdd(mb.pairCount, 1);
     if (slot < mb.pairCap) mb.pairs[slot] = make_float4(c2, __int_as_float(a), __int_as_float(b), __int_as_float(ko));
     else atomicOr(err, kErrOverflow);
