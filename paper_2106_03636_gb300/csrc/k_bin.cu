@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(kGridRows) k_grid_sums(int nRows, const int* _
 __global__ void __launch_bounds__(kGridRows) k_grid(int nRows, const int* __restrict__ rowCnt, const int* __restrict__ rowMin,
                                                     const int* __restrict__ rowMax, const GeomConst* __restrict__ G,
                                                     RowGrid* __restrict__ grid, int* __restrict__ nfBlockStart,
-                                                    int nfBlock, const int* __restrict__ sums,
+                                                    int* __restrict__ nfBlockRow, int nfBlock,
+                                                    const int* __restrict__ sums,
                                                     int* __restrict__ totals) {
   __shared__ int ws[3][kGridRows / 32], base[3][kGridRows / 32];
   const int R = blockIdx.x * kGridRows + threadIdx.x;
@@ -259,6 +260,8 @@ __global__ void __launch_bounds__(kGridRows) k_grid(int nRows, const int* __rest
     g.cellBase = x[1];
     grid[R] = g;
     nfBlockStart[R] = x[2];
+    if (nfBlockRow)
+      for (int b = 0; b < v[2]; ++b) nfBlockRow[x[2] + b] = R;
     if (R == nRows - 1) {
       totals[0] = x[0] + v[0];
       totals[1] = x[1] + v[1];
@@ -601,12 +604,13 @@ void launch_row_reduce(const TFDesc* tfs, int nTF, int* tileStats, int* rowCnt, 
 }
 
 void launch_grid(int nRows, const int* rowCnt, const int* rowMin, const int* rowMax, const GeomConst* G,
-                 RowGrid* grid, int* nfBlockStart, int nfBlock, int* totals, cudaStream_t st) {
+                 RowGrid* grid, int* nfBlockStart, int* nfBlockRow, int nfBlock, int* totals, cudaStream_t st) {
   if (nRows <= 0) return;
   int* sums = totals + 4;
   const int nb = grid_blocks(nRows);
   k_grid_sums<<<nb, kGridRows, 0, st>>>(nRows, rowCnt, rowMin, rowMax, G, nfBlock, sums);
-  k_grid<<<nb, kGridRows, 0, st>>>(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, nfBlock, sums, totals);
+  k_grid<<<nb, kGridRows, 0, st>>>(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, nfBlockRow, nfBlock, sums,
+                               totals);
   g_launch_count += 2;
 }
 

@@ -245,41 +245,31 @@ __device__ inline void nf_view(const ZView& V, const ZRow& gu, const ZRow& gd, i
   }
 }
 
-// First index of a[0, n) with a[i] > v, searched by the whole warp: 32 probes
-// a step, 3-4 dependent loads where a binary search takes 13-18 (all lanes
-// must call it; every lane gets the result).
-__device__ inline int warp_upper_bound(const int* __restrict__ a, int n, int v) {
-  const int lane = threadIdx.x & 31;
-  int lo = 0, hi = n;  // answer in [lo, hi]
-  while (hi > lo) {
-    const int step = (hi - lo + 31) / 32;
-    const int i = lo + lane * step;  // ascending probes
-    const unsigned m = __ballot_sync(0xffffffffu, i < hi && a[i] <= v);
-    const int k = __popc(m);  // probes at or below v
-    if (k == 0) return lo;
-    lo += (k - 1) * step + 1;
-    hi = min(hi, lo + step - 1);
-  }
-  return lo;
-}
+// Threads of the NeighboursFinder kernels resident on an SM: 40 registers a
+// thread with some 190 bytes of spills, for twelve warps a scheduler.  They
+// wait for candidates more than they compute: 1 ms frame (20.3 M clusters) 0.90
+// ms with 64 registers, 0.80 with 48, 0.75 with 40, 0.77 with 32; across a
+// missing row (10 collisions) 0.21 -> 0.18 ms.
+constexpr int kNFResident = 1536;
 
 // K4: one thread per hit in the drift order of its row; blocks of kB hits
-// tile the rows (nfBlockStart, built for the same block size, maps a block to
-// its row, looked up once per block).  The hits of a warp are neighbours in
-// drift, so their candidates on an adjacent row are one run of 40-50 hits and
-// every lane's share of it is about equal: 8 candidates a side to test, against
-// 11 in the cells with the second cell row scanned by the few lanes that
-// reach it.  A hit next to a row flagged dense takes the cells.
+// tile the rows (nfBlockRow, built for the same block size, names a block's
+// row).  The hits of a warp are neighbours in drift, so their candidates on an
+// adjacent row are one run of 40-50 hits and every lane's share of it is about
+// equal: 8 candidates a side to test, against 11 in the cells with the second
+// cell row scanned by the few lanes that reach it.  A hit next to a row flagged dense takes the cells.
 // Against the search in the cells: 1 ms frame (20.3 M clusters) 1.80 -> 0.94
-// ms, 32 orbits (59 M) 6.02 -> 3.63 ms; the views cost 0.16 and 0.56 ms.
+// ms, 32 orbits (59 M) 6.02 -> 3.63 ms (0.75 and 2.75 with kNFResident); the views
+// cost 0.20 and 0.62 ms.
 template <int kB>
-__global__ void __launch_bounds__(kB) k_neighbours_view(const RowGrid* __restrict__ grid,
-                                                        const int* __restrict__ nfBlockStart, int nRows,
+__global__ void __launch_bounds__(kB, kNFResident / kB) k_neighbours_view(const RowGrid* __restrict__ grid,
+                                                        const int* __restrict__ nfBlockStart,
+                                                        const int* __restrict__ nfBlockRow, int nRows,
                                                         const int* __restrict__ cellStart,
                                                         const int2* __restrict__ syz, const GeomConst* __restrict__ G,
                                                         ZView zv, int* __restrict__ upRaw, int* __restrict__ dnRaw) {
   if ((int)blockIdx.x >= nfBlockStart[nRows]) return;  // launched with an upper bound of blocks
-  const int R = warp_upper_bound(nfBlockStart, nRows + 1, blockIdx.x) - 1;
+  const int R = nfBlockRow[blockIdx.x];
   const ZRow g = zv.rows[R];
   const int q = (blockIdx.x - nfBlockStart[R]) * kB + threadIdx.x;
   if (q >= g.count) return;
@@ -545,14 +535,15 @@ __device__ inline void gap_view(const ZView& V, const ZRow& gu, const ZRow& gd, 
 // warps work.  Rows flagged dense take the cells.
 // 10 collisions of a 1 ms frame with 5 % of the clusters lost: 1.36 -> 0.21 ms.
 template <int kB>
-__global__ void __launch_bounds__(kB) k_neighbours_gap(const int* __restrict__ nfBlockStart, int nRows,
+__global__ void __launch_bounds__(kB, kNFResident / kB) k_neighbours_gap(const int* __restrict__ nfBlockStart,
+                                                       const int* __restrict__ nfBlockRow, int nRows,
                                                        const RowGrid* __restrict__ grid,
                                                        const int* __restrict__ cellStart,
                                                        const int2* __restrict__ syz, const GeomConst* __restrict__ G,
                                                        ZView zv, int* __restrict__ upRaw, int* __restrict__ dnRaw) {
   if ((int)blockIdx.x >= nfBlockStart[nRows]) return;  // launched with an upper bound of blocks
   __shared__ int s_pos[kB], s_cnt[kB / 32];
-  const int R = warp_upper_bound(nfBlockStart, nRows + 1, blockIdx.x) - 1;
+  const int R = nfBlockRow[blockIdx.x];
   const int r = (R % kRowsPerTF) % kNRow;
   if (r < 1 || r > kNRow - 2) return;
   const ZRow g = zv.rows[R];
@@ -867,15 +858,15 @@ void launch_lower_bounds(const int* list, const int* nListDev, const int* keys, 
 }
 
 void launch_neighbours(int nfBlocks, int hitsPerBlock, bool stage, const RowGrid* grid, const int* nfBlockStart,
-                       int nRows, const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw,
-                       int* dnRaw, unsigned* err, cudaStream_t st, unsigned inject) {
+                       const int* nfBlockRow, int nRows, const int* cellStart, const int2* syz, const GeomConst* G,
+                       ZView zv, int* upRaw, int* dnRaw, unsigned* err, cudaStream_t st, unsigned inject) {
   if (nfBlocks > 0) {
 #define O2TPC_NF(B)                                                                                                  \
   if (stage)                                                                                                         \
     k_neighbours_staged<B><<<nfBlocks, B, 0, st>>>(grid, nfBlockStart, nRows, cellStart, syz, G, upRaw, dnRaw, err,  \
                                                    inject);                                                          \
   else                                                                                                               \
-    k_neighbours_view<B><<<nfBlocks, B, 0, st>>>(grid, nfBlockStart, nRows, cellStart, syz, G, zv, upRaw, dnRaw)
+    k_neighbours_view<B><<<nfBlocks, B, 0, st>>>(grid, nfBlockStart, nfBlockRow, nRows, cellStart, syz, G, zv, upRaw, dnRaw)
     if (hitsPerBlock == 64) {
       O2TPC_NF(64);
     } else if (hitsPerBlock == 256) {
@@ -888,12 +879,12 @@ void launch_neighbours(int nfBlocks, int hitsPerBlock, bool stage, const RowGrid
   }
 }
 
-void launch_neighbours_gap(int nfBlocks, int hitsPerBlock, const int* nfBlockStart, const RowGrid* grid, int nRows,
-                           const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw, int* dnRaw,
+void launch_neighbours_gap(int nfBlocks, int hitsPerBlock, const int* nfBlockStart, const int* nfBlockRow,
+                           const RowGrid* grid, int nRows, const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw, int* dnRaw,
                            cudaStream_t st) {
   if (nfBlocks > 0) {
 #define O2TPC_GAP(B) \
-  k_neighbours_gap<B><<<nfBlocks, B, 0, st>>>(nfBlockStart, nRows, grid, cellStart, syz, G, zv, upRaw, dnRaw)
+  k_neighbours_gap<B><<<nfBlocks, B, 0, st>>>(nfBlockStart, nfBlockRow, nRows, grid, cellStart, syz, G, zv, upRaw, dnRaw)
     if (hitsPerBlock == 64) O2TPC_GAP(64);
     else if (hitsPerBlock == 256) O2TPC_GAP(256);
     else O2TPC_GAP(128);

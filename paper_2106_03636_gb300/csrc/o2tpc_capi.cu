@@ -345,7 +345,7 @@ void tune_cache_store(Ctx* c);
 // arrays as any other; the grid's block map is rebuilt for the chosen NF
 // shape before the real NeighboursFinder launch.
 void autotune(Ctx* c, int n, int nRows, const int* rowCnt, const int* rowMin, const int* rowMax, RowGrid* grid,
-              int* nfBlockStart, int* totals, int4* bucket, int* cellStart, int2* syz, int* sorig, int* gscratch,
+              int* nfBlockStart, int* nfBlockRow, int* totals, int4* bucket, int* cellStart, int2* syz, int* sorig, int* gscratch,
               ZRow* zrow, unsigned* err) {
   cudaStream_t st = c->stream;
   const GeomConst* G = c->dGeom;
@@ -370,10 +370,10 @@ void autotune(Ctx* c, int n, int nRows, const int* rowCnt, const int* rowMin, co
   const ZView zv{zrow, reinterpret_cast<const char*>(bucket)};
   for (int i = 0; i < 6; ++i) {
     const int hb = kNF[i % 3];
-    launch_grid(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, hb, totals, st);
+    launch_grid(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, nfBlockRow, hb, totals, st);
     const int blocks = n / hb + nRows + 1;
     CK(cudaEventRecord(en[i][0], st));
-    launch_neighbours(blocks, hb, i >= 3, grid, nfBlockStart, nRows, cellStart, syz, G, zv, up, up + n, err, st);
+    launch_neighbours(blocks, hb, i >= 3, grid, nfBlockStart, nfBlockRow, nRows, cellStart, syz, G, zv, up, up + n, err, st);
     CK(cudaEventRecord(en[i][1], st));
   }
   CK(cudaEventSynchronize(en[5][1]));
@@ -402,7 +402,7 @@ void autotune(Ctx* c, int n, int nRows, const int* rowCnt, const int* rowMin, co
   c->tune.tuned = 1;
   c->tune.tuned_on_clusters = n;
   tune_cache_store(c);
-  launch_grid(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, c->tune.nf_hits_per_block, totals, st);
+  launch_grid(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, nfBlockRow, c->tune.nf_hits_per_block, totals, st);
 }
 
 // What the download and the kept stages need from a pipeline run.
@@ -661,12 +661,13 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   int* rowMax = dalloc<int>(M, nRows);
   RowGrid* grid = dalloc<RowGrid>(M, nRows + 1);
   int* nfBlockStart = dalloc<int>(M, nRows + 1);
+  int* nfBlockRow = dalloc<int>(M, n / 64 + nRows + 1);
   int* totals = dalloc<int>(M, 4 + 3 * grid_blocks(nRows));
   launch_ingest_stats(dTF, dTiles, nTiles, tileSize, G, tileStats, dErr, st);
   CKL();
   launch_row_reduce(dTF, B, tileStats, rowCnt, rowMin, rowMax, st);
   CKL();
-  launch_grid(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, c->tune.nf_hits_per_block, totals, st);
+  launch_grid(nRows, rowCnt, rowMin, rowMax, G, grid, nfBlockStart, nfBlockRow, c->tune.nf_hits_per_block, totals, st);
   CKL();
   const long long cellsMax = (long long)n / kHitsPerCell + 46ll * nRows + 1;
   CK(cudaEventRecord(c->evs[1], st));
@@ -680,7 +681,7 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   launch_cell_sort(n, nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, c->tune.sort_threads_per_row);
   ZRow* zrow = dalloc<ZRow>(M, nRows);
   if ((c->cfg.flags & O2TPC_FLAG_AUTOTUNE) && !c->tune.tuned && n >= (1 << 20))
-    autotune(c, n, nRows, rowCnt, rowMin, rowMax, grid, nfBlockStart, totals, bucket, cellStart, syz, sorig, gscratch,
+    autotune(c, n, nRows, rowCnt, rowMin, rowMax, grid, nfBlockStart, nfBlockRow, totals, bucket, cellStart, syz, sorig, gscratch,
              zrow, dErr);
   else
     launch_zorder(nRows, grid, rowMax, cellStart, syz, zrow, bucket, st);
@@ -697,11 +698,11 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   int* scratch = dalloc<int>(M, scan_scratch_ints((long long)n + 8) + (nRows + 8) * 2 / 4096 + 64);
   const int nfB = c->tune.nf_hits_per_block;
   const int nfBlocksMax = n / nfB + nRows + 1;
-  launch_neighbours(nfBlocksMax, nfB, c->tune.nf_staged != 0, grid, nfBlockStart, nRows, cellStart, syz, G, zv,
+  launch_neighbours(nfBlocksMax, nfB, c->tune.nf_staged != 0, grid, nfBlockStart, nfBlockRow, nRows, cellStart, syz, G, zv,
                     upRaw, dnRaw, dErr, st, c->cfg.debug_inject);
   CKL();
   if (c->cfg.flags & O2TPC_FLAG_ROW_STEP2) {
-    launch_neighbours_gap(nfBlocksMax, nfB, nfBlockStart, grid, nRows, cellStart, syz, G, zv, upRaw, dnRaw, st);
+    launch_neighbours_gap(nfBlocksMax, nfB, nfBlockStart, nfBlockRow, grid, nRows, cellStart, syz, G, zv, upRaw, dnRaw, st);
     CKL();
   }
   CK(cudaEventRecord(c->evs[3], st));

@@ -63,6 +63,7 @@ size_t graph_carve(GraphArena& A, char* base) {
   take(A.rowMax, k.nRows);
   take(A.grid, k.nRows + 1);
   take(A.nfBlockStart, k.nRows + 1);
+  take(A.nfBlockRow, n / 64 + k.nRows + 1);
   take(A.totals, 4 + 3 * grid_blocks(k.nRows));
   take(A.cellStart, k.cellsCap + 1);
   take(A.gscratch, k.cellsCap);
@@ -175,17 +176,18 @@ void graph_enqueue(const GraphArena& A, const GeomConst* G, int nfBlock, bool nf
   // A1-A4
   launch_ingest_stats(A.tfs, A.tiles, k.nTilesCap, k.tileSize, G, A.tileStats, A.err, st);
   launch_row_reduce(A.tfs, k.BCap, A.tileStats, A.rowCnt, A.rowMin, A.rowMax, st);
-  launch_grid(k.nRows, A.rowCnt, A.rowMin, A.rowMax, G, A.grid, A.nfBlockStart, nfBlock, A.totals, st);
+  launch_grid(k.nRows, A.rowCnt, A.rowMin, A.rowMax, G, A.grid, A.nfBlockStart, A.nfBlockRow, nfBlock, A.totals,
+              st);
   launch_row_scatter(A.tfs, A.tiles, k.nTilesCap, k.tileSize, G, A.tileStats, A.grid, A.bucket, st);
   launch_cell_sort(n, k.nRows, A.grid, A.bucket, A.cellStart, A.syz, A.sorig, A.gscratch, A.totals, st, sortThreads);
   launch_zorder(k.nRows, A.grid, A.rowMax, A.cellStart, A.syz, A.zrow, A.bucket, st);
   const ZView zv{A.zrow, reinterpret_cast<const char*>(A.bucket)};
   // A5-A7
-  launch_neighbours(n / nfBlock + k.nRows + 1, nfBlock, nfStage, A.grid, A.nfBlockStart, k.nRows, A.cellStart, A.syz, G, zv,
-                    A.upRaw, A.dnRaw, A.err, st);
+  launch_neighbours(n / nfBlock + k.nRows + 1, nfBlock, nfStage, A.grid, A.nfBlockStart, A.nfBlockRow,
+                    k.nRows, A.cellStart, A.syz, G, zv, A.upRaw, A.dnRaw, A.err, st);
   if (rowStep2)
-    launch_neighbours_gap(n / nfBlock + k.nRows + 1, nfBlock, A.nfBlockStart, A.grid, k.nRows, A.cellStart, A.syz, G, zv,
-                          A.upRaw, A.dnRaw, st);
+    launch_neighbours_gap(n / nfBlock + k.nRows + 1, nfBlock, A.nfBlockStart, A.nfBlockRow, A.grid, k.nRows,
+                          A.cellStart, A.syz, G, zv, A.upRaw, A.dnRaw, st);
   launch_clean(n, &C->n, A.upRaw, A.dnRaw, A.up, A.dn, A.flag, st);
   launch_ballot_count(n, &C->n, A.flag, A.tileCnt, A.tileOff, &C->nTl, k.tlCap, &C->overflow, A.scratch, st);
   launch_ballot_compact(n, &C->n, A.flag, A.tileOff, A.starts, k.tlCap, &C->overflow, st);

@@ -24,7 +24,7 @@ struct GraphArena {
   int* tileStats;
   int *rowCnt, *rowMin, *rowMax;
   RowGrid* grid;
-  int* nfBlockStart;
+  int *nfBlockStart, *nfBlockRow;
   int* totals;
   int* cellStart;
   int* gscratch;

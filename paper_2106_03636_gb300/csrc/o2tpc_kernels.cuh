@@ -19,13 +19,14 @@ void launch_ingest_stats(const TFDesc* tfs, const int2* tiles, int nTiles, int t
                          int* tileStats, unsigned* err, cudaStream_t st);
 void launch_row_reduce(const TFDesc* tfs, int nTF, int* tileStats, int* rowCnt, int* rowMin, int* rowMax,
                        cudaStream_t st);
-// totals: 4 ints, then 3 * grid_blocks(nRows) of scratch.
+// totals: 4 ints, then 3 * grid_blocks(nRows) of scratch.  nfBlockRow (may be
+// null): the row of every NeighboursFinder block, n / nfBlock + nRows + 1 ints.
 int grid_blocks(int nRows);
 // Clusters per ingest tile of a batch of n clusters.
 constexpr int kTileMin = 8192, kTileMax = 65536;
 int ingest_tile(long long n);
 void launch_grid(int nRows, const int* rowCnt, const int* rowMin, const int* rowMax, const GeomConst* G,
-                 RowGrid* grid, int* nfBlockStart, int nfBlock, int* totals, cudaStream_t st);
+                 RowGrid* grid, int* nfBlockStart, int* nfBlockRow, int nfBlock, int* totals, cudaStream_t st);
 void launch_row_scatter(const TFDesc* tfs, const int2* tiles, int nTiles, int tileSize, const GeomConst* G,
                         const int* tileStats, const RowGrid* grid, int4* bucket, cudaStream_t st);
 // n: clusters (or their capacity), by which the rows' counters are sized.
@@ -43,12 +44,12 @@ void launch_zorder(int nRows, const RowGrid* grid, const int* rowMax, const int*
 // slab copies may read it); err collects kErrTimeout.  inject: the context's
 // debug_inject bits (bit 0: staged slabs armed but not copied, short waits).
 void launch_neighbours(int nfBlocks, int hitsPerBlock, bool stage, const RowGrid* grid, const int* nfBlockStart,
-                       int nRows, const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw,
-                       int* dnRaw, unsigned* err, cudaStream_t st, unsigned inject = 0);
+                       const int* nfBlockRow, int nRows, const int* cellStart, const int2* syz, const GeomConst* G,
+                       ZView zv, int* upRaw, int* dnRaw, unsigned* err, cudaStream_t st, unsigned inject = 0);
 // Row step 2: links across one missing row for the hits that found no
 // adjacent-row pair (after launch_neighbours, with the same blocks).
-void launch_neighbours_gap(int nfBlocks, int hitsPerBlock, const int* nfBlockStart, const RowGrid* grid, int nRows,
-                           const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw, int* dnRaw,
+void launch_neighbours_gap(int nfBlocks, int hitsPerBlock, const int* nfBlockStart, const int* nfBlockRow,
+                           const RowGrid* grid, int nRows, const int* cellStart, const int2* syz, const GeomConst* G, ZView zv, int* upRaw, int* dnRaw,
                            cudaStream_t st);
 // Data-dependent sizes are read by the kernels from device memory (nDev,
 // the fields of Counts); the host-side n of a launcher only sizes its grid:

@@ -153,7 +153,7 @@ extern "C" int o2tpc_sort_tf_static(const o2tpc_tf* tf, double vdrift_cm_us, int
   RowGrid* grid = reinterpret_cast<RowGrid*>(row_grid);
   launch_ingest_stats(P.tf, P.tiles, d.nTiles, kStaticTile, P.geom, P.tileStats, P.err, st);
   launch_row_reduce(P.tf, 1, P.tileStats, P.rowCnt, P.rowMin, P.rowMax, st);
-  launch_grid(kRowsPerTF, P.rowCnt, P.rowMin, P.rowMax, P.geom, grid, P.nfBlockStart, kNFBlock, P.totals, st);
+  launch_grid(kRowsPerTF, P.rowCnt, P.rowMin, P.rowMax, P.geom, grid, P.nfBlockStart, nullptr, kNFBlock, P.totals, st);
   launch_row_scatter(P.tf, P.tiles, d.nTiles, kStaticTile, P.geom, P.tileStats, grid, P.bucket, st);
   launch_cell_sort(n, kRowsPerTF, grid, P.bucket, cell_start, reinterpret_cast<int2*>(sorted_yz), sorted_orig,
                    P.cellScratch, P.totals, st);
