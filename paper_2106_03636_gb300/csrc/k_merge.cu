@@ -193,7 +193,7 @@ __device__ inline bool chi2_5(const float* d, const float* M, float cut, float& 
 }
 
 // One thread per outer border end A: all B candidates of the neighbour edge.
-__global__ void __launch_bounds__(128) k_merge_pairs(SectorTrackBufs sb, const GeomConst* __restrict__ G,
+__global__ void __launch_bounds__(128, 1) k_merge_pairs(SectorTrackBufs sb, const GeomConst* __restrict__ G,
                                                      MergeBufs mb, unsigned* __restrict__ err) {
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= mb.cnt->nSt) return;
@@ -546,7 +546,7 @@ __device__ inline int chain_tail(int head, const int* __restrict__ next, int* ns
 // With one loop over a track's segments, hits loaded a step ahead and the
 // cluster lists in k_track_clusters: 1 ms frame 0.69 -> 0.33 ms (+ 0.05 for the
 // lists), 32 orbits 1.74 -> 0.84 (+ 0.14), 3 collisions 0.345 -> 0.12.
-__global__ void __launch_bounds__(128) k_final_refit(const int* __restrict__ nHeadsDev,
+__global__ void __launch_bounds__(128, 1) k_final_refit(const int* __restrict__ nHeadsDev,
                                                                const int* __restrict__ heads, SectorTrackBufs sb,
                                                                MergeBufs mb, const int2* __restrict__ syz,
                                                                const GeomConst* __restrict__ G, int forceFp64,

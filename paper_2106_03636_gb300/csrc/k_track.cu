@@ -112,6 +112,10 @@ __device__ inline int warp_take(int* counter, bool want) {
 // is one chain's latency, and the fit follows the links itself.
 // 1 ms frame (664 k tracklets) 0.57 -> 0.34 ms + 0.15 for the walk and the order,
 // 32 orbits 1.57 -> 0.89 + 0.5.
+// One CTA per SM as the least for the fits (here, the refits, the sector fits, the
+// merger's pairs): they are bound by their chains of arithmetic, so registers
+// (72-96 against 68-72) count for more than warps; 16 orbits: chain and refit
+// 1.73 -> 1.68 ms, sector fits 0.65 -> 0.63 ms; with 64 registers 1.80 and 0.68.
 constexpr int kChainOrdered = 40000;
 
 __global__ void __launch_bounds__(256) k_tl_walk(const int* __restrict__ nTlDev, const int* __restrict__ starts,
@@ -128,7 +132,7 @@ __global__ void __launch_bounds__(256) k_tl_walk(const int* __restrict__ nTlDev,
   tb.nasc[k] = n;
 }
 
-__global__ void __launch_bounds__(128) k_tl_chain(const int* __restrict__ nTlDev, int* __restrict__ counter,
+__global__ void __launch_bounds__(128, 1) k_tl_chain(const int* __restrict__ nTlDev, int* __restrict__ counter,
                                                   const int* __restrict__ perm, const int* __restrict__ starts,
                                                   const int* __restrict__ up, const RowGrid* __restrict__ grid,
                                                   int nRows, const int2* __restrict__ syz,
@@ -206,7 +210,7 @@ __global__ void __launch_bounds__(128) k_tl_chain(const int* __restrict__ nTlDev
 // order of their length; hits are loaded one step ahead.
 // 1 ms frame (664 k tracklets): 0.64 -> 0.49 ms, 32 orbits 1.85 -> 1.43 ms (27 of
 // 32 lanes active, 20 in plain order; now 65 % issue-active).
-__global__ void __launch_bounds__(128) k_tl_refit(const int* __restrict__ nTlDev, int* __restrict__ counter,
+__global__ void __launch_bounds__(128, 1) k_tl_refit(const int* __restrict__ nTlDev, int* __restrict__ counter,
                                                             const int* __restrict__ perm, const int2* __restrict__ syz,
                                                             const GeomConst* __restrict__ G, TrackletBufs tb) {
   const float zunit = G->zunit, bzc = G->bzc;
@@ -1096,7 +1100,7 @@ __global__ void __launch_bounds__(128, 6) k_segments_write(const int* __restrict
 // Alone with few tracks (one collision of a sector) 164 -> 110 us: its time is the
 // chain of steps; 32 orbits 0.99 ms as in a global order by length, without its
 // scattered results.
-__global__ void __launch_bounds__(128) k_sector_fit(const int* __restrict__ nStDev, int* __restrict__ counter,
+__global__ void __launch_bounds__(128, 1) k_sector_fit(const int* __restrict__ nStDev, int* __restrict__ counter,
                                                               const int* __restrict__ perm, TrackletBufs tb, const GeomConst* __restrict__ G,
                                                               SectorTrackBufs sb) {
   const float zunit = G->zunit, bzc = G->bzc;
