@@ -362,9 +362,9 @@ __global__ void __launch_bounds__(kScatterT) k_row_scatter(const TFDesc* __restr
 // by input index).  Cell counters live in shared memory when the row has at
 // most smemCells cells, else in the global scratch.  smemCells is sized for rows
 // of 2.5 times the average (launch_cell_sort), so that more CTAs share an SM
-// than with room for the largest (48 KB): 1 ms frame 0.62 -> 0.41 ms, 32 orbits 2.08 ->
+// than with room for the largest (47.5 KB): 1 ms frame 0.62 -> 0.41 ms, 32 orbits 2.08 ->
 // 1.63 ms, 3 collisions 112 -> 56 us.
-constexpr int kSmemCells = 12288;  // at most: 48 KB
+constexpr int kSmemCells = 12160;  // at most: 47.5 KB, so that with the kernel's own 144 bytes a CTA stays within 48 KB
 constexpr int kRegSort = 8;
 
 template <int kT>
