@@ -153,7 +153,8 @@ typedef struct {
   int32_t nf_hits_per_block;     /* NeighboursFinder: hits (threads) per block of a
                                     pad row: 64, 128 (default) or 256             */
   int32_t sort_threads_per_row;  /* cell sort: threads per pad row: 128, 256
-                                    (default) or 512                              */
+                                    or 512 (default: by the rows' size, and
+                                    o2tpc_tuning then says 256)                   */
   /* Captured path (0: off): batches of at most graph_max_tfs TFs (0: 64) and
    * graph_max_clusters clusters run as ONE CUDA graph launch - the whole
    * pipeline captured once and replayed, no host synchronisation inside -

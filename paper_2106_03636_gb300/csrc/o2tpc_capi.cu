@@ -168,6 +168,7 @@ struct Ctx {
   GeomConst* dGeom = nullptr;
   Counts* dCounts = nullptr;  // sizes of the running regular-path batch
   GeomConst hGeom{};
+  int sortThreads = 0;  // cell sort: configured or tuned threads per row, 0: by the rows' size
   std::thread worker;
   std::mutex mu;
   std::condition_variable cvWork, cvDone;
@@ -397,6 +398,7 @@ void autotune(Ctx* c, int n, int nRows, const int* rowCnt, const int* rowMin, co
   for (auto& r : en)
     for (auto& e : r) cudaEventDestroy(e);
   c->tune.sort_threads_per_row = kSort[bs];
+  c->sortThreads = kSort[bs];
   c->tune.nf_hits_per_block = kNF[bn % 3];
   c->tune.nf_staged = bn >= 3 ? 1 : 0;
   c->tune.tuned = 1;
@@ -518,7 +520,7 @@ bool run_captured(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, 
   const int slot = c->graphSlot;
   if (c->graphDlRecorded[slot]) CK(cudaStreamWaitEvent(st, c->graphDl[slot], 0));
   if (c->graphExec[0] && (c->graphNf != c->tune.nf_hits_per_block * 2 + c->tune.nf_staged ||
-                          c->graphSort != c->tune.sort_threads_per_row)) {
+                          c->graphSort != c->sortThreads)) {
     for (auto& e : c->graphExec) {
       if (e) cudaGraphExecDestroy(e);
       e = nullptr;
@@ -531,7 +533,7 @@ bool run_captured(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, 
       cudaGraph_t g = nullptr;
       CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
       const long long before = g_launch_count;
-      graph_enqueue(As, c->dGeom, c->tune.nf_hits_per_block, c->tune.nf_staged != 0, c->tune.sort_threads_per_row,
+      graph_enqueue(As, c->dGeom, c->tune.nf_hits_per_block, c->tune.nf_staged != 0, c->sortThreads,
                     (c->cfg.flags & O2TPC_FLAG_FORCE_FP64) ? 1 : 0, st,
                     (c->cfg.flags & O2TPC_FLAG_COOP_SEARCH) != 0, (c->cfg.flags & O2TPC_FLAG_ROW_STEP2) != 0);
       const cudaError_t ce = cudaStreamEndCapture(st, &g);
@@ -550,7 +552,7 @@ bool run_captured(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, 
       cudaGraphDestroy(g);
     }
     c->graphNf = c->tune.nf_hits_per_block * 2 + c->tune.nf_staged;
-    c->graphSort = c->tune.sort_threads_per_row;
+    c->graphSort = c->sortThreads;
   }
   g_launch_count = c->graphKernels;
   CK(cudaEventRecord(c->evs[0], st));
@@ -678,7 +680,7 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   int* sorig = dalloc<int>(M, n);
   launch_row_scatter(dTF, dTiles, nTiles, tileSize, G, tileStats, grid, bucket, st);
   CKL();
-  launch_cell_sort(n, nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, c->tune.sort_threads_per_row);
+  launch_cell_sort(n, nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, c->sortThreads);
   ZRow* zrow = dalloc<ZRow>(M, nRows);
   if ((c->cfg.flags & O2TPC_FLAG_AUTOTUNE) && !c->tune.tuned && n >= (1 << 20))
     autotune(c, n, nRows, rowCnt, rowMin, rowMax, grid, nfBlockStart, nfBlockRow, totals, bucket, cellStart, syz, sorig, gscratch,
@@ -990,6 +992,7 @@ void tune_cache_load(Ctx* c) {
       c->tune.nf_hits_per_block = nf;
       c->tune.nf_staged = staged ? 1 : 0;
       c->tune.sort_threads_per_row = sort;
+      c->sortThreads = sort;
       c->tune.tuned = 1;
     }
   }
@@ -1488,6 +1491,7 @@ int o2tpc_create(const o2tpc_config* cfg, o2tpc_ctx** out) {
   x->cfg = c;
   x->tune.nf_hits_per_block = c.nf_hits_per_block;
   x->tune.sort_threads_per_row = c.sort_threads_per_row;
+  x->sortThreads = cfg ? cfg->sort_threads_per_row : 0;
   x->tune.nf_staged = c.nf_staged ? 1 : 0;
   if (c.flags & O2TPC_FLAG_AUTOTUNE) tune_cache_load(x);
   x->traceCopies = std::getenv("O2TPC_TRACE_COPIES") != nullptr;

@@ -32,7 +32,7 @@ void launch_row_scatter(const TFDesc* tfs, const int2* tiles, int nTiles, int ti
 // n: clusters (or their capacity), by which the rows' counters are sized.
 void launch_cell_sort(int n, int nRows, const RowGrid* grid, const int4* bucket, int* cellStart, int2* syz, int* sorig,
                       int* gscratch, const int* totals, cudaStream_t st,
-                      int threadsPerRow = 256);
+                      int threadsPerRow = 0);
 
 // The drift-ordered views (ZRow) of all rows, written over the bucket records
 // of the rows (used up by the cell sort; their memory stays the view's).
