@@ -896,17 +896,27 @@ struct TlPlaces {
   }
 };
 
-// Consecutive tracklets a warp takes at once: 32, fewer when there are too few
-// for every warp of the grid.
+// CTAs an SM of the two passes: all resident, so that the tracklets in flight are
+// one run of consecutive ones; fewer from kSegMany tracklets on, where the words
+// and coordinates of that run no longer stay in L2.  (Grids of 12 CTAs an SM and
+// groups of 32 ran over the TF twice: selection of 16 orbits (1.1 M tracklets) 1.88 ->
+// 1.67 ms, 96 orbits (6.4 M) 13.1 -> 11.6 ms, with 7 and 4 CTAs 10.2; of 16
+// orbits with 7 and 4 1.70 ms.)
+constexpr int kSegCountCtas = 10, kSegWriteCtas = 6, kSegCountMany = 7, kSegWriteMany = 4, kSegMany = 3000000;
+
+// Consecutive tracklets a warp takes at once: 8 (selection of 16 orbits 1.92 ms
+// with 32, 1.69 with 8, 1.79 with 2), fewer when there are too few for every warp
+// of the grid.
+constexpr int kSegGroup = 8;
 __device__ inline int segment_group(int nTl) {
   const int warps = gridDim.x * (blockDim.x >> 5);
-  return min(32, max(1, (nTl + warps - 1) / warps));
+  return min(kSegGroup, max(1, (nTl + warps - 1) / warps));
 }
 
 // K8b: count pass; also keeps the ownership bits (in row order) for the write
 // pass, which then reads no ownership words.
-__global__ void __launch_bounds__(128, 10) k_segments_count(const int* __restrict__ nTlDev, OwnCtx o, TrackletBufs tb,
-                                                        int* __restrict__ nSeg, int* __restrict__ nSegHits,
+__global__ void __launch_bounds__(128, kSegCountCtas) k_segments_count(const int* __restrict__ nTlDev, OwnCtx o,
+                                                        TrackletBufs tb, int* __restrict__ nSeg, int* __restrict__ nSegHits,
                                                         unsigned* __restrict__ ownBits) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, nTl = *nTlDev;
@@ -988,7 +998,7 @@ __global__ void __launch_bounds__(128, 10) k_segments_count(const int* __restric
 // gather the coordinates and input indices of their hits for the fits.  A
 // tracklet has at most 27 segments, kept or not (they lie 6 rows apart): a lane
 // each for their table entries.
-__global__ void __launch_bounds__(128, 6) k_segments_write(const int* __restrict__ nTlDev, TrackletBufs tb,
+__global__ void __launch_bounds__(128, kSegWriteCtas) k_segments_write(const int* __restrict__ nTlDev, TrackletBufs tb,
                                                         const unsigned* __restrict__ ownBits,
                                                         const int* __restrict__ segPos,
                                                         const int* __restrict__ segHitPos,
@@ -1240,15 +1250,16 @@ void launch_ownership(int nTl, const int* nTlDev, int nSec, const RowGrid* grid,
 }
 
 namespace {
-// warps of 1 to 32 tracklets, up to twelve blocks of four warps an SM
-int segment_blocks(int nTl) { return std::min((nTl + 3) / 4, pass_grid().sms * 12); }
+int segment_blocks(int nTl, int perSM, int perSMMany) {
+  return std::min((nTl + 3) / 4, pass_grid().sms * (nTl < kSegMany ? perSM : perSMMany));
+}
 }  // namespace
 
 void launch_segments_count(int nTl, const int* nTlDev, const int* secBegin, const int* wide, const void* w,
                            TrackletBufs tb, int* nSeg, int* nSegHits, unsigned* ownBits, cudaStream_t st) {
   if (nTl > 0) {
-    k_segments_count<<<segment_blocks(nTl), 128, 0, st>>>(nTlDev, OwnCtx{secBegin, wide, const_cast<void*>(w)}, tb,
-                                                          nSeg, nSegHits, ownBits);
+    k_segments_count<<<segment_blocks(nTl, kSegCountCtas, kSegCountMany), 128, 0, st>>>(
+        nTlDev, OwnCtx{secBegin, wide, const_cast<void*>(w)}, tb, nSeg, nSegHits, ownBits);
     ++g_launch_count;
   }
 }
@@ -1257,8 +1268,8 @@ void launch_segments_write(int nTl, const int* nTlDev, TrackletBufs tb, const un
                            const int* segHitPos, const int2* syz, const int* sorig, SectorTrackBufs sb, int capSt,
                            int capHits, cudaStream_t st) {
   if (nTl > 0) {
-    k_segments_write<<<segment_blocks(nTl), 128, 0, st>>>(nTlDev, tb, ownBits, segPos, segHitPos, syz, sorig, sb,
-                                                          capSt, capHits);
+    k_segments_write<<<segment_blocks(nTl, kSegWriteCtas, kSegWriteMany), 128, 0, st>>>(
+        nTlDev, tb, ownBits, segPos, segHitPos, syz, sorig, sb, capSt, capHits);
     ++g_launch_count;
   }
 }
