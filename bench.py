@@ -73,14 +73,14 @@ STAGE_BYTES = {
 # workload, valid while the kernel's sources hash to the recorded value;
 # otherwise the line says null.
 MEASURED_TRAFFIC = {
-    # the following passes: one-pass DRAM counters of a single kernel on the
+    # the following passes: DRAM counters of the single kernels on the
     # 1 ms frame (19.70 M clusters at the same 50 kHz density), scaled by the
     # cluster count (x 241.96 / 19.70) to a launch on the 128-orbit TF
-    ("k_tl_follow<1>", "full_tf"): {"bytes": (1256651008 + 318376704) * 241.96 / 19.70,
-                                    "sources_sha256_16": "c51eb7e4024de7bf",
+    ("k_tl_follow<1>", "full_tf"): {"bytes": (2390308000 + 363173888) * 241.96 / 19.70,
+                                    "sources_sha256_16": "5dee0b74b98df2b5",
                                     "sources": ["k_track.cu", "o2tpc_internal.cuh"]},
-    ("k_tl_follow<-1>", "full_tf"): {"bytes": (1249804288 + 240405760) * 241.96 / 19.70,
-                                     "sources_sha256_16": "c51eb7e4024de7bf",
+    ("k_tl_follow<-1>", "full_tf"): {"bytes": (2240776000 + 251170560) * 241.96 / 19.70,
+                                     "sources_sha256_16": "5dee0b74b98df2b5",
                                      "sources": ["k_track.cu", "o2tpc_internal.cuh"]},
 }
 
@@ -99,7 +99,7 @@ def measured_traffic(kernel: str, workload: str):
 
 
 # kernels (or single-kernel steps) the roofline line can name
-ROOF_KERNELS = {"tl_out": "k_tl_follow<1>", "tl_in": "k_tl_follow<-1>", "neighbours": "k_neighbours",
+ROOF_KERNELS = {"tl_out": "k_tl_follow<1>", "tl_in": "k_tl_follow<-1>", "neighbours": "k_neighbours_view",
                 "refit": "k_final_refit", "sort": "k_row_scatter+k_cell_sort", "selection": "k_ownership+k_segments",
                 "sector_fit": "k_sector_fit", "merge": "k_merge_*"}
 PATH_BYTES = 65.0
@@ -218,13 +218,12 @@ def run_raw(args, rank, world, local):
                        "clusters_out": int(nc), "l2": "inputs larger than L2 (no flush)",
                        "parallelism": f"replicas x{world}"},
             "clusters_per_s": world * nc / (ms / 1e3),
-            "roofline": {"bound": "hbm", "kernel": "o2tpc_clusterize (k_clu_keys + k_clu_flags + compaction + "
-                                                    "k_clu_records)",
+            "roofline": {"bound": "hbm", "kernel": "o2tpc_clusterize (k_clu_tile twice + scan)",
                          "achieved": alg / (ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                          "frac": alg / (ms / 1e3) / 1e9 / peak, "traffic": None, "peak_kind": peak_kind,
                          "bytes_per_digit": alg / d.n},
             "tracked_after": {"status": res["status"], "tracks": res["n_tracks"]},
-            "clocks": clk.summary(), "gpu_launches": 9 * args.steps}
+            "clocks": clk.summary(), "gpu_launches": 3 * args.steps}
     if rank == 0:
         print(json.dumps(line), flush=True)
     if world > 1:
