@@ -77,10 +77,10 @@ MEASURED_TRAFFIC = {
     # 1 ms frame (19.70 M clusters at the same 50 kHz density), scaled by the
     # cluster count (x 241.96 / 19.70) to a launch on the 128-orbit TF
     ("k_tl_follow<1>", "full_tf"): {"bytes": (2390308000 + 363173888) * 241.96 / 19.70,
-                                    "sources_sha256_16": "5dee0b74b98df2b5",
+                                    "sources_sha256_16": "3f3b31b4c299e15c",
                                     "sources": ["k_track.cu", "o2tpc_internal.cuh"]},
     ("k_tl_follow<-1>", "full_tf"): {"bytes": (2240776000 + 251170560) * 241.96 / 19.70,
-                                     "sources_sha256_16": "5dee0b74b98df2b5",
+                                     "sources_sha256_16": "3f3b31b4c299e15c",
                                      "sources": ["k_track.cu", "o2tpc_internal.cuh"]},
 }
 

@@ -854,8 +854,10 @@ __global__ void k_ownership(const int* __restrict__ nTlDev, OwnCtx o, TrackletBu
 // other with a lane per hit, the next one's lists on their way: lists, rows and
 // results are read and written as whole lines, 32 random words in flight.
 // (With a thread per tracklet the write pass ran with 6.5 of 32 lanes active.)
-// 1 ms frame: count 0.30 -> 0.31, write with the coordinate gather 0.55 -> 0.32
-// ms; one sector's frame 39 + 57 -> 8 + 8 us; 32 orbits 0.76 + 1.44 -> 0.95 + 1.35.
+// Count and write with the coordinate gather, against a thread per tracklet, with groups
+// of 32 (groups of 8 take another tenth off): 1 ms frame 0.30 + 0.55 -> 0.31 + 0.32 ms, one
+// sector's frame 39 + 57 -> 8 + 8 us, 32 orbits 0.76 + 1.44 -> 0.95 + 1.35 ms.  128 orbits:
+// 3.0 + 5.7 -> 4.6 + 6.1 ms with groups of 8.
 constexpr int kSegWords = kOwnWords;
 
 // Slot of the tracklet's j-th hit in row order (nd of its nh hits are inward).
