@@ -572,8 +572,16 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
     __syncthreads();
     bL = bR;
   }
-  // too far apart: the searches of this row's neighbourhood take the cells
-  if (__syncthreads_or(far) && threadIdx.x == 0) zrow[blockIdx.x].flags = kZNFCells | kZFollowCells;
+  // too far apart: the view becomes the sorted order itself (distance 0
+  // throughout, which the row's own hits are taken from), and the searches into
+  // this row take the cells
+  if (__syncthreads_or(far)) {
+    for (int h = threadIdx.x; h < g.count; h += kZThreads) {
+      yz[h] = syz[g.start + h];
+      idx[h] = 0;
+    }
+    if (threadIdx.x == 0) zrow[blockIdx.x].flags = kZNFCells | kZFollowCells;
+  }
 }
 
 // ------------------------------------------------------------- launchers
