@@ -43,13 +43,7 @@ __device__ inline bool decode(const TFDesc& t, const RawCluster& w, const GeomCo
   int s, r;
   bool ok = true;
   if (t.format == 1) {
-    uint32_t w0 = w.a, w1 = w.b, w2 = w.c;
-    uint32_t pad = w1 & 0xFFFFu;
-    r = (int)(w2 & 0xFFu);
-    s = (int)((w2 >> 8) & 0xFFu);
-    if (s >= kNSec || r >= kNRow || w0 > 0x3FFFFFFFu) { ok = false; s = 0; r = 0; }
-    yu = (int)pad - 32 * G->npads[r];
-    zu = (int)w0;
+    ok = decode_fixed(w.a, w.b, w.c, G->npads, s, r, yu, zu);
   } else {
     s = (int)(w.c & 0xFFu);
     r = (int)((w.c >> 8) & 0xFFu);
@@ -184,9 +178,7 @@ __device__ inline RowGrid row_grid(int R, int nRows, const int* __restrict__ row
   g.count = n;
   if (n > 0) {
     g.nz = min(max((n + kHitsPerCell * g.ny - 1) / (kHitsPerCell * g.ny), 1), kMaxNz);
-    // 1 .. 2^31 + 1 units over 1 .. 2^20 cells
-    const unsigned range = (unsigned)rowMax[R] - (unsigned)rowMin[R] + 1u;
-    g.cz = (int)((range + (unsigned)g.nz - 1u) / (unsigned)g.nz);
+    g.cz = cell_height(rowMin[R], rowMax[R], g.nz);
     g.zmin = rowMin[R];
   }
   return g;

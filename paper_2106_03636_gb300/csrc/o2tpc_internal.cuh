@@ -173,6 +173,29 @@ __host__ __device__ inline int floordiv_i32(int a, int b) {
   return (q * b > a) ? q - 1 : q;
 }
 
+// A stored record of the fixed format (its three words): sector, row and
+// integer coordinates.  False for a sector, row or time that does not exist;
+// the record is then filed under row 0 with its time cut to the 30 bits of a
+// valid one, so that every coordinate a row sees stays within +-2^30 (a batch
+// runs to its end before the host reads the error word).
+__host__ __device__ inline bool decode_fixed(uint32_t w0, uint32_t w1, uint32_t w2, const int* npads, int& s, int& r,
+                                             int& yu, int& zu) {
+  r = (int)(w2 & 0xFFu);
+  s = (int)((w2 >> 8) & 0xFFu);
+  const bool ok = s < kNSec && r < kNRow && w0 <= 0x3FFFFFFFu;
+  if (!ok) s = r = 0;
+  yu = (int)(w1 & 0xFFFFu) - 32 * npads[r];
+  zu = (int)(w0 & 0x3FFFFFFFu);
+  return ok;
+}
+
+// Drift units of a cell of a row with extremes zmin and zmax and nz cells:
+// ceil(range / nz) for the 1 .. 2^31 + 1 units of a row, without the sum that
+// leaves 32 bits for a larger range.
+__host__ __device__ inline int cell_height(int zmin, int zmax, int nz) {
+  return (int)(((unsigned)zmax - (unsigned)zmin) / (unsigned)nz + 1u);
+}
+
 __device__ inline int cell_iy(const RowGrid& g, int npads, int yu) {
   int half = 32 * npads;
   int iy = floordiv_i32(yu + half, kCellY);
