@@ -725,10 +725,14 @@ __device__ int refit_chain64(int head, int tail, const SectorTrackBufs& sb, cons
 // ~50 instructions for one track against ~180 for 32, so the lines cross at
 // about 608 * 180 / 50.
 // One track of the 1 ms frame: 0.94 -> 0.36 ms; four of 32 orbits 0.49 -> 0.18.
+// All tracks of a small frame forced to FP64, refit step with a block of four
+// warps per 128 tracks of the frame -> four blocks an SM: 57 tracks 5.8 -> 0.53
+// ms, 478 11.5 -> 0.58, 1844 11.7 -> 1.20 (one block an SM 1.50, two 1.30, eight
+// 1.75); a thread each: 2923 tracks 1.64.
 constexpr int kWarpRefit64 = 2048;
 __global__ void __launch_bounds__(128) k_final_refit64(const int* __restrict__ heads, SectorTrackBufs sb, MergeBufs mb,
                                                        const int2* __restrict__ syz, const GeomConst* __restrict__ G,
-                                                       OutBufs ob) {
+                                                       OutBufs ob, int sms) {
   const int nf = *ob.nFallback;
   if (nf <= kWarpRefit64) {
     const int lane = threadIdx.x & 31;
@@ -737,8 +741,10 @@ __global__ void __launch_bounds__(128) k_final_refit64(const int* __restrict__ h
     r.j = lane < 25 ? lane % 5 : 4;
     r.ii = max(r.i, r.j);
     r.jj = min(r.i, r.j);
-    // warps of one block come last: neighbours in the queue go to different SMs
-    for (int q = blockIdx.x + gridDim.x * (threadIdx.x >> 5); q < nf; q += gridDim.x * (blockDim.x >> 5)) {
+    // warps of one block come last: neighbours in the queue go to different
+    // SMs; the first warp of each block of an SM to another quarter
+    const int w = ((threadIdx.x >> 5) + blockIdx.x / sms) & 3;
+    for (int q = blockIdx.x + gridDim.x * w; q < nf; q += gridDim.x * 4) {
       const int t = ob.fallback[q];
       const int head = heads[t];
       int nseg;
@@ -852,18 +858,25 @@ void launch_final_refit(int nHeads, const int* nHeadsDev, int nSt, const int* he
                         MergeBufs mb, const int2* syz, const TFDesc* tfs, const GeomConst* G, int forceFp64,
                         int* counter, int* perm, OutBufs ob, cudaStream_t st) {
   if (nHeads > 0) {
-    static int sms = 0, perSm = 0;
-    if (sms == 0) {
+    struct Sizes {
+      int sms = 0, perSm = 0;
+    };
+    static const Sizes z = [] {
+      Sizes v;
       int dev = 0;
       cudaGetDevice(&dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, k_final_refit, 128, 0);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v.perSm, k_final_refit, 128, 0);
+      cudaDeviceGetAttribute(&v.sms, cudaDevAttrMultiProcessorCount, dev);
+      return v;
+    }();
+    const int sms = std::max(z.sms, 1);
     k_track_clusters<<<std::min((nSt + 7) / 8, sms * 8), 256, 0, st>>>(sb, mb, tfs, ob.off, ob.cl);
     launch_length_order(nHeads, nHeadsDev, ob.off, true, perm, st);
-    const int nb = std::min((nHeads + 127) / 128, sms * std::max(perSm, 1));
+    const int nb = std::min((nHeads + 127) / 128, sms * std::max(z.perSm, 1));
     k_final_refit<<<nb, 128, 0, st>>>(nHeadsDev, heads, sb, mb, syz, G, forceFp64, counter, perm, ob);
-    k_final_refit64<<<std::min((nHeads + 127) / 128, sms * 4), 128, 0, st>>>(heads, sb, mb, syz, G, ob);
+    // a CTA a track as long as there are CTAs: how many tracks are queued, and
+    // with it the form, is known on the device alone
+    k_final_refit64<<<std::min(nHeads, sms * 4), 128, 0, st>>>(heads, sb, mb, syz, G, ob, sms);
     g_launch_count += 3;
   }
 }
