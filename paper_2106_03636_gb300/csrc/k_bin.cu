@@ -352,27 +352,20 @@ __global__ void __launch_bounds__(kScatterT) k_row_scatter(const TFDesc* __restr
 // K3b: one CTA per row.  Counting sort of the row's bucket by cell into the
 // final arrays, then input order restored inside every cell (insertion sort
 // by input index).  Cell counters live in shared memory when the row has at
-// most smemCells cells, else in the global scratch.  smemCells is sized for rows
-// of 2.5 times the average (launch_cell_sort), so that more CTAs share an SM
-// than with room for the largest (47.5 KB): 1 ms frame 0.62 -> 0.41 ms, 32 orbits 2.08 ->
-// 1.63 ms, 3 collisions 112 -> 56 us.
+// most smemCells cells.  smemCells is sized for rows of 2.5 times the average
+// (launch_cell_sort), so that more CTAs share an SM than with room for the
+// largest (47.5 KB): 1 ms frame 0.62 -> 0.41 ms, 32 orbits 2.08 -> 1.63 ms, 3
+// collisions 112 -> 56 us.  Rows of more cells count in the global scratch;
+// those of more than farCells, which only frames with few filled rows have, are
+// left to k_cell_sort_large.
 constexpr int kSmemCells = 12160;  // at most: 47.5 KB, so that with the kernel's own 144 bytes a CTA stays within 48 KB
+constexpr int kLargeCells = 11520;  // with k_cell_sort_large's list and statics within 48 KB too
 constexpr int kRegSort = 8;
 
-template <int kT>
-__global__ void __launch_bounds__(kT) k_cell_sort(const RowGrid* __restrict__ grid, const int4* __restrict__ bucket,
-                                                   int* __restrict__ cellStart, int2* __restrict__ syz,
-                                                   int* __restrict__ sorig, int* __restrict__ gscratch,
-                                                   int smemCells) {
-  extern __shared__ int s_cnt[];
+__device__ inline void sort_row(const RowGrid& g, int* cnt, const int4* __restrict__ bucket,
+                                int* __restrict__ cellStart, int2* __restrict__ syz, int* __restrict__ sorig) {
   __shared__ int s_carry;
-  const RowGrid g = grid[blockIdx.x];
-  if (g.count == 0) {
-    for (int c = threadIdx.x; c < g.ny * g.nz; c += blockDim.x) cellStart[g.cellBase + c] = g.start;
-    return;
-  }
   const int nc = g.ny * g.nz;
-  int* cnt = (nc <= smemCells) ? s_cnt : (gscratch + g.cellBase);
   for (int c = threadIdx.x; c < nc; c += blockDim.x) cnt[c] = 0;
   __syncthreads();
   const int4* bk = bucket + g.start;
@@ -465,6 +458,49 @@ __global__ void __launch_bounds__(kT) k_cell_sort(const RowGrid* __restrict__ gr
       sorig[j + 1] = ko;
       syz[j + 1] = kv;
     }
+  }
+}
+
+template <int kT>
+__global__ void __launch_bounds__(kT) k_cell_sort(const RowGrid* __restrict__ grid, const int4* __restrict__ bucket,
+                                                   int* __restrict__ cellStart, int2* __restrict__ syz,
+                                                   int* __restrict__ sorig, int* __restrict__ gscratch,
+                                                   int smemCells, int farCells) {
+  extern __shared__ int s_cnt[];
+  const RowGrid g = grid[blockIdx.x];
+  const int nc = g.ny * g.nz;
+  if (g.count == 0) {
+    for (int c = threadIdx.x; c < nc; c += blockDim.x) cellStart[g.cellBase + c] = g.start;
+    return;
+  }
+  if (nc > farCells) return;
+  sort_row(g, nc <= smemCells ? s_cnt : gscratch + g.cellBase, bucket, cellStart, syz, sorig);
+}
+
+// The rows of more than minCells cells, by resident CTAs of 512 threads with
+// the largest counters: each looks for them among every gridDim.x-th row, a row
+// a thread.  One sector filled, 2.1 M clusters in 152 rows: sort 0.39 -> 0.19 ms
+// (CTAs of 128 threads that count in the global scratch, one an SM, before),
+// 4.2 M 0.88 -> 0.38 ms.
+template <int kT>
+__global__ void __launch_bounds__(kT) k_cell_sort_large(int nRows, const RowGrid* __restrict__ grid,
+                                                         const int4* __restrict__ bucket, int* __restrict__ cellStart,
+                                                         int2* __restrict__ syz, int* __restrict__ sorig,
+                                                         int* __restrict__ gscratch, int minCells) {
+  extern __shared__ int s_cnt[];
+  __shared__ int s_rows[kT], s_n;
+  for (int r0 = blockIdx.x; r0 < nRows; r0 += kT * gridDim.x) {
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const long long r = r0 + (long long)threadIdx.x * gridDim.x;
+    if (r < nRows && grid[r].count > 0 && grid[r].ny * grid[r].nz > minCells) s_rows[atomicAdd(&s_n, 1)] = (int)r;
+    __syncthreads();
+    for (int k = 0; k < s_n; ++k) {
+      const RowGrid g = grid[s_rows[k]];
+      sort_row(g, g.ny * g.nz <= kLargeCells ? s_cnt : gscratch + g.cellBase, bucket, cellStart, syz, sorig);
+      __syncthreads();  // the counters are no longer in use
+    }
+    __syncthreads();  // nor the list
   }
 }
 
@@ -664,13 +700,35 @@ void launch_cell_sort(int n, int nRows, const RowGrid* grid, const int4* bucket,
     const long long want = 5ll * n / (2ll * kHitsPerCell * nRows) + 128;
     const int cells = (int)std::min<long long>(std::max<long long>(want, 512), kSmemCells);
     const size_t smem = sizeof(int) * cells;
-    if (threadsPerRow == 128)
-      k_cell_sort<128><<<nRows, 128, smem, st>>>(grid, bucket, cellStart, syz, sorig, gscratch, cells);
-    else if (threadsPerRow == 512)
-      k_cell_sort<512><<<nRows, 512, smem, st>>>(grid, bucket, cellStart, syz, sorig, gscratch, cells);
-    else
-      k_cell_sort<256><<<nRows, 256, smem, st>>>(grid, bucket, cellStart, syz, sorig, gscratch, cells);
-    ++g_launch_count;
+    // Rows of four times the counters of a TF that holds all n clusters (ten
+    // times its average) are k_cell_sort_large's; its launch (2-3 us) is left out
+    // where a single filled sector would not have them.  (All rows past the
+    // counters there: one sector the same, but a graph with room for 64 TFs given
+    // one of 20 M clusters 10.23 -> 10.35 ms, eight of 0.7 M 1 % slower.)
+    const int farCells = (int)std::min<long long>(
+        std::max<long long>(5ll * n / (2ll * kHitsPerCell * kRowsPerTF) + 128, 512) * 4, INT_MAX);
+    const bool large = n / (kNRow * kHitsPerCell) > farCells;
+    auto sort = [&](auto kernel, int threads) {
+      kernel<<<nRows, threads, smem, st>>>(grid, bucket, cellStart, syz, sorig, gscratch, cells,
+                                           large ? farCells : INT_MAX);
+      ++g_launch_count;
+    };
+    if (threadsPerRow == 128) sort(k_cell_sort<128>, 128);
+    else if (threadsPerRow == 512) sort(k_cell_sort<512>, 512);
+    else sort(k_cell_sort<256>, 256);
+    if (large) {
+      constexpr int kT = 512;
+      static const int ctas = [] {
+        int dev = 0, sms = 0, per = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cell_sort_large<kT>, kT, sizeof(int) * kLargeCells);
+        return std::max(sms, 1) * std::max(per, 1);
+      }();
+      k_cell_sort_large<kT><<<std::min(ctas, nRows), kT, sizeof(int) * kLargeCells, st>>>(
+          nRows, grid, bucket, cellStart, syz, sorig, gscratch, farCells);
+      ++g_launch_count;
+    }
   }
   k_cell_sentinel<<<1, 1, 0, st>>>(cellStart, totals);
   ++g_launch_count;
