@@ -172,7 +172,7 @@ __device__ inline RowGrid row_grid(int R, int nRows, const int* __restrict__ row
   RowGrid g{};
   if (R >= nRows) return g;  // no hits, no cells
   const int n = rowCnt[R];
-  g.ny = max(1, (64 * G->npads[(R % kRowsPerTF) % kNRow] + kCellY - 1) / kCellY);
+  g.ny = cells_y(G->npads[(R % kRowsPerTF) % kNRow]);
   g.nz = 1;
   g.cz = 1;
   g.count = n;
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kScatterT) k_row_scatter(const TFDesc* __restr
           g.cz = s_cz[lr];
           g.nz = s_nz[lr];
           const int npads = s_npads[lr % kNRow];
-          g.ny = max(1, (64 * npads + kCellY - 1) / kCellY);
+          g.ny = cells_y(npads);
           const int iy = cell_iy(g, npads, yu);
           const int iz = cell_iz_floor(zu, g);  // zu >= zmin of its row: 0..nz-1
           const int slot = atomicAdd(&s_cur[lr], 1);
@@ -525,6 +525,9 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
   ZRow z{};
   z.start = g.start;
   z.count = g.count;
+  z.cellBase = g.cellBase;
+  z.cz = g.cz;
+  z.flags = g.nz << kZnz;
   if (g.count == 0) {
     if (threadIdx.x == 0) zrow[blockIdx.x] = z;
     return;
@@ -608,7 +611,7 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
       yz[h] = syz[g.start + h];
       idx[h] = 0;
     }
-    if (threadIdx.x == 0) zrow[blockIdx.x].flags = kZNFCells | kZFollowCells;
+    if (threadIdx.x == 0) zrow[blockIdx.x].flags = z.flags | kZNFCells | kZFollowCells;
   }
 }
 

@@ -592,7 +592,9 @@ __global__ void __launch_bounds__(128, 7) k_tl_follow_coop(const int* __restrict
 }
 
 // The same passes with the per-lane search in the drift-ordered views (rows
-// flagged dense: in the cells).  Bound by the latency of the dependent chain of a row
+// flagged dense: in the cells, whose place is in the view's row table: with the
+// cells' own table as one more dependent load a sector of 2.1 M clusters took
+// 0.77 + 1.24 ms, now 0.67 + 1.23).  Bound by the latency of the dependent chain of a row
 // step (row table -> bin starts -> candidates -> update) and by its ~450
 // instructions.  Only what the next reader needs survives a step: the
 // direction parameters and the row of the last accepted state (with kKeep the
@@ -616,8 +618,8 @@ constexpr int kFollowBatch = 8;
 
 template <int kDir, bool kKeep>
 __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
-    k_tl_follow(const int* __restrict__ nTlDev, int* __restrict__ counter, const RowGrid* __restrict__ grid,
-                const int* __restrict__ cellStart, const int2* __restrict__ syz, const GeomConst* __restrict__ G,
+    k_tl_follow(const int* __restrict__ nTlDev, int* __restrict__ counter, const int* __restrict__ cellStart,
+                const int2* __restrict__ syz, const GeomConst* __restrict__ G,
                 ZView zv, TrackletBufs tb) {
   constexpr bool kWhole = kKeep && kDir < 0;
   __shared__ float s_last[kWhole ? 20 : 1][128];
@@ -725,7 +727,13 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
         int zlo, zhi;
         if (g.count > 0 && search_window(st, yref, zref, izunit, angErr, P, zlo, zhi)) {
           if (g.flags & kZFollowCells) {
-            const RowGrid gc = grid[Rs + r];
+            RowGrid gc;
+            gc.count = g.count;
+            gc.cellBase = g.cellBase;
+            gc.ny = cells_y(G->npads[r]);
+            gc.nz = g.flags >> kZnz;
+            gc.cz = g.cz;
+            gc.zmin = g.zmin;
             int ylo, yhi, iy0, iy1, iz0, iz1;
             window_y(P, ylo, yhi);
             if (cell_range(gc, G->npads[r], ylo, yhi, zlo, zhi, iy0, iy1, iz0, iz1))
@@ -1223,7 +1231,7 @@ void launch_tracklets(int nTl, const int* nTlDev, int* workCounter, const int* s
   if (coopSearch) {
     k_tl_follow_coop<1><<<blocks(g.out), 128, 0, st>>>(nTlDev, workCounter + 1, grid, cellStart, syz, G, tb);
   } else {
-    k_tl_follow<1, false><<<blocks(g.out), 128, 0, st>>>(nTlDev, workCounter + 1, grid, cellStart, syz, G, zv, tb);
+    k_tl_follow<1, false><<<blocks(g.out), 128, 0, st>>>(nTlDev, workCounter + 1, cellStart, syz, G, zv, tb);
   }
   mark(1);
   launch_length_order(nTl, nTlDev, tb.nasc, false, perm, st);
@@ -1232,9 +1240,9 @@ void launch_tracklets(int nTl, const int* nTlDev, int* workCounter, const int* s
   if (coopSearch) {
     k_tl_follow_coop<-1><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, grid, cellStart, syz, G, tb);
   } else if (keepState) {
-    k_tl_follow<-1, true><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, grid, cellStart, syz, G, zv, tb);
+    k_tl_follow<-1, true><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, cellStart, syz, G, zv, tb);
   } else {
-    k_tl_follow<-1, false><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, grid, cellStart, syz, G, zv, tb);
+    k_tl_follow<-1, false><<<blocks(g.in), 128, 0, st>>>(nTlDev, workCounter + 3, cellStart, syz, G, zv, tb);
   }
   mark(3);
   g_launch_count += 5;

@@ -89,8 +89,8 @@ struct ZRow {
   int zmin;
   int nzb;      // drift bins
   float zinv;   // bins per drift unit
-  int flags;    // kZNFCells, kZFollowCells
-  int pad0, pad1;
+  int flags;    // kZNFCells, kZFollowCells, nz << kZnz
+  int cellBase, cz;  // as RowGrid (with nz): the following of a flagged row reads no other table
 };
 // Rows so dense that the cells hold fewer candidates than the drift window:
 // bit 0 for the NeighboursFinder's window, bit 1 for the following's.  Both are
@@ -98,7 +98,7 @@ struct ZRow {
 // more than 32 k hits): such a row's view is its sorted order with distances of
 // 0 and has no bin starts, so that a row's own hits are read from its view
 // whatever the flags say, and a flagged row is searched in its cells alone.
-enum : int { kZNFCells = 1, kZFollowCells = 2 };
+enum : int { kZNFCells = 1, kZFollowCells = 2, kZnz = 8 };
 constexpr int kZShortRow = 65535;  // hits of a row with 16-bit bin starts, at most
 
 // The drift-ordered views of a batch: row tables and the record memory.
@@ -187,6 +187,12 @@ __host__ __device__ inline bool decode_fixed(uint32_t w0, uint32_t w1, uint32_t 
   yu = (int)(w1 & 0xFFFFu) - 32 * npads[r];
   zu = (int)(w0 & 0x3FFFFFFFu);
   return ok;
+}
+
+// Cells of a row across its pads.
+__host__ __device__ inline int cells_y(int npads) {
+  const int c = (64 * npads + kCellY - 1) / kCellY;
+  return c > 1 ? c : 1;
 }
 
 // Drift units of a cell of a row with extremes zmin and zmax and nz cells:
