@@ -512,10 +512,7 @@ __global__ void __launch_bounds__(kT) k_cell_sort_large(int nRows, const RowGrid
 // counted, scanned and scattered by itself in shared memory, its output range
 // is its input range, and the writes stay inside it.  Bound by memory: 8
 // bytes read (twice, the second time from L2), 10 + 2 per bin written per hit.
-constexpr int kZBins = 4096, kZThreads = 256;
-// Units, 0.5 cm at 2.58 cm/us: half a following window.  1 cm: following 3 %, the
-// NeighboursFinder 6 % slower on 16 orbits; 2 cm: 18 and 30 %.
-constexpr int kZBinWidth = 62;
+constexpr int kZThreads = 256;
 __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict__ grid, const int* __restrict__ rowMax,
                                                       const int* __restrict__ cellStart, const int2* __restrict__ syz,
                                                       ZRow* __restrict__ zrow, int4* __restrict__ bucket) {
@@ -534,7 +531,7 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
   }
   const float range = (float)((unsigned)rowMax[blockIdx.x] - (unsigned)g.zmin) + 1.f;
   z.zmin = g.zmin;
-  z.nzb = max(1, min(min((int)(range * (1.f / kZBinWidth)), g.count), g.nz * (kZBins - 96)));
+  z.nzb = drift_bins(range, g.count, g.nz);
   z.zinv = (float)z.nzb / range;
   // expected hits of a whole row in a window (plus the bins' own width)
   // against ~10 in the cells that cover it

@@ -14,6 +14,7 @@ using namespace o2tpc;
 extern "C" int t_decode_fixed(const uint32_t* w, const int* npads, int* o) {
   return decode_fixed(w[0], w[1], w[2], npads, o[0], o[1], o[2], o[3]) ? 1 : 0;
 }
+extern "C" int t_drift_bins(float range, int count, int nz) { return drift_bins(range, count, nz); }
 extern "C" int t_cell_height(int zmin, int zmax, int nz) { return cell_height(zmin, zmax, nz); }
 """
 
@@ -59,3 +60,14 @@ def test_cell_height(lib, zmin, zmax):
     for nz in (1, 2, 3, 7, 1000, 8214, (1 << 20) - 1, 1 << 20):
         want = (zmax - zmin + nz) // nz
         assert lib.t_cell_height(zmin, zmax, nz) & 0xFFFFFFFF == want & 0xFFFFFFFF
+
+
+@pytest.mark.parametrize("nz", [1, 2, 1000, 536870, 536871, 1 << 20])
+def test_drift_bins(lib, nz):
+    """The least of 62 units a bin, a bin a hit and 4000 a cell row, also past 2^31 of these."""
+    lib.t_drift_bins.argtypes = [ctypes.c_float, ctypes.c_int, ctypes.c_int]
+    for count in (1, 100, 40000000):
+        for rng in (1.0, 61.0, 6200.0, 2.0 ** 31):
+            got = lib.t_drift_bins(rng, count, nz)
+            want = max(1, min(int(np.float32(rng) * np.float32(1 / 62)), count, nz * 4000))
+            assert abs(got - want) <= (rng > 2 ** 24)
