@@ -319,7 +319,7 @@ typedef struct {
  * and the centre of gravity of the 3 x 3 cells around it, rounded half up in
  * 1/64 pad and 1/64 time bin.  Runs on `stream` (a cudaStream_t, NULL for the
  * default stream) with scratch from the stream-ordered allocator and returns
- * when the records are written.  *n_clusters: the number of peaks (also when
+ * when the records are written (the buffer may overlap the digits' arrays).  *n_clusters: the number of peaks (also when
  * it exceeds cap).  Returns O2TPC_OK, O2TPC_EINVAL (null pointers, misaligned
  * records, unsorted or out-of-range digits), O2TPC_ETOOBIG (n >= 2^31, or more
  * peaks than cap: nothing written), O2TPC_ENOMEM, O2TPC_ECUDA. */

@@ -235,6 +235,12 @@ __global__ void __launch_bounds__(kCluThreads) k_clu_tile(CluIn d, int* __restri
   }
 }
 
+// Whether two ranges of bytes share any.
+static bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + nb && y < x + na;
+}
+
 }  // namespace o2tpc
 
 using namespace o2tpc;
@@ -282,8 +288,25 @@ extern "C" int o2tpc_clusterize(const o2tpc_digits* d, void* records, uint64_t c
     if (herr & kErrInput) { rc = O2TPC_EINVAL; break; }
     *n_clusters = (uint64_t)total;
     if ((uint64_t)total > cap) { rc = O2TPC_ETOOBIG; break; }
-    if (total > 0)
-      k_clu_tile<true><<<nt, kCluThreads, 0, st>>>(in, nullptr, tileOff, static_cast<uint8_t*>(records), nullptr);
+    if (total > 0) {
+      // pass 2 reads the digits again: records that are to take their place are
+      // written beside them first
+      const size_t bytes = 12 * (size_t)total, m = (size_t)n;
+      uint8_t *dst = static_cast<uint8_t*>(records), *beside = nullptr;
+      if (overlap(dst, bytes, d->sector, m) || overlap(dst, bytes, d->row, m) || overlap(dst, bytes, d->pad, m) ||
+          overlap(dst, bytes, d->time, 4 * m) || overlap(dst, bytes, d->adc, 2 * m)) {
+        if (cudaMallocAsync(reinterpret_cast<void**>(&beside), bytes, st) != cudaSuccess) {
+          cudaGetLastError();
+          rc = O2TPC_ENOMEM;
+          break;
+        }
+      }
+      k_clu_tile<true><<<nt, kCluThreads, 0, st>>>(in, nullptr, tileOff, beside ? beside : dst, nullptr);
+      if (beside) {
+        if (cudaMemcpyAsync(dst, beside, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) rc = O2TPC_ECUDA;
+        cudaFreeAsync(beside, st);
+      }
+    }
     if (cudaGetLastError() != cudaSuccess) rc = O2TPC_ECUDA;
   } while (false);
   cudaFreeAsync(base, st);
