@@ -153,8 +153,7 @@ typedef struct {
   int32_t nf_hits_per_block;     /* NeighboursFinder: hits (threads) per block of a
                                     pad row: 64, 128 (default) or 256             */
   int32_t sort_threads_per_row;  /* cell sort: threads per pad row: 128, 256
-                                    or 512 (default: by the rows' size, and
-                                    o2tpc_tuning then says 256)                   */
+                                    or 512 (default: by the rows' size)           */
   /* Captured path (0: off): batches of at most graph_max_tfs TFs (0: 64) and
    * graph_max_clusters clusters run as ONE CUDA graph launch - the whole
    * pipeline captured once and replayed, no host synchronisation inside -
@@ -188,7 +187,8 @@ typedef struct {
   int32_t tuned;                 /* 1 once the autotuner has chosen               */
   int32_t nf_hits_per_block;
   int32_t nf_staged;
-  int32_t sort_threads_per_row;
+  int32_t sort_threads_per_row;  /* of the last batch, when no shape was asked for
+                                    or chosen (256 before the first)              */
   int32_t tuned_on_clusters;     /* size of the batch it tuned on                 */
   float nf_ms[6];                /* 64, 128, 256 hits per block; L1 then staged   */
   float sort_ms[3];              /* 128, 256, 512 threads per row                 */

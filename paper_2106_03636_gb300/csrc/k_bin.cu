@@ -686,17 +686,22 @@ void launch_row_scatter(const TFDesc* tfs, const int2* tiles, int nTiles, int ti
   }
 }
 
+// No shape asked for: by the hits of an average row.  Short rows idle large
+// CTAs in every barrier; of long rows, fewer at once stay in L2 between
+// the two reads.  Sort of 3 collisions (240 a row) 96 / 109 / 131 us with
+// 128 / 256 / 512 threads, 10 collisions (750) 217 / 225 / 248 us, 1 ms frame
+// (3700) 1.13 / 1.06 / 1.08 ms, 16 orbits (5400) 2.25 / 1.95 / 1.96, 48 orbits
+// (16 k) 7.66 / 7.12 / 6.09, 96 orbits (32 k) 13.6 / 12.2 / 11.5.
+int cell_sort_threads(int n, int nRows, int asked) {
+  if (asked != 0) return asked;
+  const int perRow = n / std::max(nRows, 1);
+  return perRow < 1000 ? 128 : perRow < 8000 ? 256 : 512;
+}
+
 void launch_cell_sort(int n, int nRows, const RowGrid* grid, const int4* bucket, int* cellStart, int2* syz, int* sorig,
                       int* gscratch, const int* totals, cudaStream_t st, int threadsPerRow) {
   if (nRows > 0) {
-    // No shape asked for: by the hits of an average row.  Short rows idle large
-    // CTAs in every barrier; of long rows, fewer at once stay in L2 between
-    // the two reads.  Sort of 3 collisions (240 a row) 96 / 109 / 131 us with
-    // 128 / 256 / 512 threads, 10 collisions (750) 217 / 225 / 248 us, 1 ms frame
-    // (3700) 1.13 / 1.06 / 1.08 ms, 16 orbits (5400) 2.25 / 1.95 / 1.96, 48 orbits
-    // (16 k) 7.66 / 7.12 / 6.09, 96 orbits (32 k) 13.6 / 12.2 / 11.5.
-    const long long perRow = n / nRows;
-    if (threadsPerRow == 0) threadsPerRow = perRow < 1000 ? 128 : perRow < 8000 ? 256 : 512;
+    threadsPerRow = cell_sort_threads(n, nRows, threadsPerRow);
     const long long want = 5ll * n / (2ll * kHitsPerCell * nRows) + 128;
     const int cells = (int)std::min<long long>(std::max<long long>(want, 512), kSmemCells);
     const size_t smem = sizeof(int) * cells;

@@ -217,6 +217,11 @@ struct Ctx {
   void* hStage = nullptr;
   size_t hStageBytes = 0;
 
+  // what the cell sort of the running batch uses, for o2tpc_get_tuning
+  void sort_shape(int threads) {
+    std::lock_guard<std::mutex> lk(mu);
+    tune.sort_threads_per_row = threads;
+  }
   void* dev_alloc(size_t bytes) { return dev_alloc_on(bytes, stream); }
   void* dev_alloc_on(size_t bytes, cudaStream_t s) {
     if (bytes == 0) bytes = 16;
@@ -554,6 +559,7 @@ bool run_captured(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, 
     c->graphNf = c->tune.nf_hits_per_block * 2 + c->tune.nf_staged;
     c->graphSort = c->sortThreads;
   }
+  c->sort_shape(cell_sort_threads(k.nCap, k.nRows, c->sortThreads));
   g_launch_count = c->graphKernels;
   CK(cudaEventRecord(c->evs[0], st));
   CK(cudaGraphLaunch(c->graphExec[slot], st));
@@ -681,6 +687,7 @@ void run_regular(Ctx* c, std::vector<std::shared_ptr<Job>>& jobs, BatchMem& M, P
   launch_row_scatter(dTF, dTiles, nTiles, tileSize, G, tileStats, grid, bucket, st);
   CKL();
   launch_cell_sort(n, nRows, grid, bucket, cellStart, syz, sorig, gscratch, totals, st, c->sortThreads);
+  c->sort_shape(cell_sort_threads(n, nRows, c->sortThreads));
   ZRow* zrow = dalloc<ZRow>(M, nRows);
   if ((c->cfg.flags & O2TPC_FLAG_AUTOTUNE) && !c->tune.tuned && n >= (1 << 20))
     autotune(c, n, nRows, rowCnt, rowMin, rowMax, grid, nfBlockStart, nfBlockRow, totals, bucket, cellStart, syz, sorig, gscratch,

@@ -29,6 +29,9 @@ void launch_grid(int nRows, const int* rowCnt, const int* rowMin, const int* row
                  RowGrid* grid, int* nfBlockStart, int* nfBlockRow, int nfBlock, int* totals, cudaStream_t st);
 void launch_row_scatter(const TFDesc* tfs, const int2* tiles, int nTiles, int tileSize, const GeomConst* G,
                         const int* tileStats, const RowGrid* grid, int4* bucket, cudaStream_t st);
+// Threads per row of the cell sort of n clusters in nRows rows: as asked for, 0:
+// by the average row.
+int cell_sort_threads(int n, int nRows, int asked);
 // n: clusters (or their capacity), by which the rows' counters are sized.
 void launch_cell_sort(int n, int nRows, const RowGrid* grid, const int4* bucket, int* cellStart, int2* syz, int* sorig,
                       int* gscratch, const int* totals, cudaStream_t st,
