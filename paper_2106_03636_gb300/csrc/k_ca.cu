@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(kB, kNFResident / kB) k_neighbours_gap(const i
   const ZRow g = zv.rows[R];
   const int q = (blockIdx.x - nfBlockStart[R]) * kB + threadIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const bool cells = (zv.rows[R + 1].flags | zv.rows[R - 1].flags) & kZNFCells;  // as k_neighbours_view
+  const bool cells = g.flags & kZNFCells;  // sorted order, as in k_neighbours_view
   const bool free = q < g.count && upRaw[cells ? g.start + q : zv.idx(g, q)] < 0;
   const unsigned m = __ballot_sync(0xffffffffu, free);
   if (lane == 0) s_cnt[w] = __popc(m);
