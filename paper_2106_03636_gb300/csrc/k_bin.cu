@@ -544,12 +544,17 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
   short* idx = reinterpret_cast<short*>(mem + 8ll * g.count);
   unsigned short* bins16 = reinterpret_cast<unsigned short*>(mem + 12ll * g.count);
   int* bins32 = reinterpret_cast<int*>(mem + 12ll * g.count);
-  bool far = false;  // an index distance beyond 16 bits
+  // A row whose view neither searches: its hits are better taken in sorted order,
+  // so that the lanes of a warp search the same cells (one sector filled,
+  // NeighboursFinder: 2.1 M clusters 17.7 ms in drift order, 16.7 so; 4.2 M 110 and
+  // 103).
+  const bool unsearched = (z.flags & (kZNFCells | kZFollowCells)) == (kZNFCells | kZFollowCells);
+  bool far = false;  // this thread met an index distance beyond 16 bits
   const float perCellRow = (float)g.cz * z.zinv * 1.0001f + 1.f;
   const int izPer = max(1, (int)((float)(kZBins - 8) / perCellRow));
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int bL = -1;  // last bin of the chunks before
-  for (int iz0 = 0; iz0 < g.nz; iz0 += izPer) {
+  for (int iz0 = 0; iz0 < g.nz && !unsearched; iz0 += izPer) {
     const int iz1 = min(iz0 + izPer, g.nz);
     const int hb = cellStart[g.cellBase + iz0 * g.ny];
     const int he = iz1 < g.nz ? cellStart[g.cellBase + iz1 * g.ny] : g.start + g.count;
@@ -600,10 +605,9 @@ __global__ void __launch_bounds__(kZThreads) k_zorder(const RowGrid* __restrict_
     __syncthreads();
     bL = bR;
   }
-  // too far apart: the view becomes the sorted order itself (distance 0
-  // throughout, which the row's own hits are taken from), and the searches into
-  // this row take the cells
-  if (__syncthreads_or(far)) {
+  // the view becomes the sorted order itself (distance 0 throughout, which the
+  // row's own hits are taken from), and the searches into this row take the cells
+  if (__syncthreads_or(far || unsearched)) {
     for (int h = threadIdx.x; h < g.count; h += kZThreads) {
       yz[h] = syz[g.start + h];
       idx[h] = 0;

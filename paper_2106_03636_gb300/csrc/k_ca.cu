@@ -279,15 +279,11 @@ __global__ void __launch_bounds__(kB, kNFResident / kB) k_neighbours_view(const 
     dnRaw[g.start + q] = -1;
     return;
   }
+  const int2 hh = zv.yz(g)[q];
+  const int h = zv.idx(g, q);
   const ZRow gu = zv.rows[R + 1], gd = zv.rows[R - 1];
-  // the hits of a block that searches the cells in sorted order, so that the
-  // lanes of a warp go through the same cells (one sector filled, 2.1 M clusters:
-  // 17.7 ms in drift order, 16.7 so; 4.2 M 110 and 103; 0.5 M 0.90 and 0.93)
-  const bool cells = (gu.flags | gd.flags) & kZNFCells;
-  const int2 hh = cells ? syz[g.start + q] : zv.yz(g)[q];
-  const int h = cells ? g.start + q : zv.idx(g, q);
   int bu = -1, bd = -1;
-  if (cells) {
+  if ((gu.flags | gd.flags) & kZNFCells) {
     const RowGrid cu = grid[R + 1], cd = grid[R - 1];
     int uy0, uy1, uz0, uz1, dy0, dy1, dz0, dz1;
     if (cell_range(cu, G->npads[r + 1], hh.x - kWinY, hh.x + kWinY, hh.y - kWinZ, hh.y + kWinZ, uy0, uy1, uz0, uz1) &&
@@ -553,8 +549,7 @@ __global__ void __launch_bounds__(kB, kNFResident / kB) k_neighbours_gap(const i
   const ZRow g = zv.rows[R];
   const int q = (blockIdx.x - nfBlockStart[R]) * kB + threadIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const bool cells = g.flags & kZNFCells;  // sorted order, as in k_neighbours_view
-  const bool free = q < g.count && upRaw[cells ? g.start + q : zv.idx(g, q)] < 0;
+  const bool free = q < g.count && upRaw[zv.idx(g, q)] < 0;
   const unsigned m = __ballot_sync(0xffffffffu, free);
   if (lane == 0) s_cnt[w] = __popc(m);
   __syncthreads();
@@ -567,7 +562,7 @@ __global__ void __launch_bounds__(kB, kNFResident / kB) k_neighbours_gap(const i
   __syncthreads();
   if ((int)threadIdx.x >= total) return;
   const int p = s_pos[threadIdx.x];
-  const int2 hh = cells ? syz[g.start + p] : zv.yz(g)[p];
+  const int2 hh = zv.yz(g)[p];
   GapBest best;
   constexpr int kSteps[3][2] = {{2, 1}, {1, 2}, {2, 2}};
 #pragma unroll 1
@@ -581,7 +576,7 @@ __global__ void __launch_bounds__(kB, kNFResident / kB) k_neighbours_gap(const i
       gap_view(zv, gu, gd, a, b, hh, best);
   }
   if (best.u >= 0) {
-    const int h = cells ? g.start + p : zv.idx(g, p);
+    const int h = zv.idx(g, p);
     upRaw[h] = best.u;
     dnRaw[h] = best.d;
   }

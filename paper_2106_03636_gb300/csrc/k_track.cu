@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(128, 7) k_tl_follow_coop(const int* __restrict
 // The same passes with the per-lane search in the drift-ordered views (rows
 // flagged dense: in the cells, whose place is in the view's row table: with the
 // cells' own table as one more dependent load a sector of 2.1 M clusters took
-// 0.77 + 1.24 ms, now 0.67 + 1.23).  Bound by the latency of the dependent chain of a row
+// 0.77 + 1.24 ms, now 0.74 + 1.23).  Bound by the latency of the dependent chain of a row
 // step (row table -> bin starts -> candidates -> update) and by its ~450
 // instructions.  Only what the next reader needs survives a step: the
 // direction parameters and the row of the last accepted state (with kKeep the
@@ -729,10 +729,12 @@ __global__ void __launch_bounds__(128, O2TPC_FOLLOW_MIN_BLOCKS)
           if (g.flags & kZFollowCells) {
             RowGrid gc;
             gc.count = g.count;
-            gc.cellBase = g.cellBase;
+            // (not with g: two more registers over the step cost every row 3 %)
+            asm volatile("ld.global.nc.v2.s32 {%0, %1}, [%2];"
+                         : "=r"(gc.cellBase), "=r"(gc.cz)
+                         : "l"(&zv.rows[Rs + r].cellBase));
             gc.ny = cells_y(G->npads[r]);
             gc.nz = g.flags >> kZnz;
-            gc.cz = g.cz;
             gc.zmin = g.zmin;
             int ylo, yhi, iy0, iy1, iz0, iz1;
             window_y(P, ylo, yhi);

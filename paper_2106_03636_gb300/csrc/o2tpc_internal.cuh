@@ -95,8 +95,8 @@ struct ZRow {
 // Rows so dense that the cells hold fewer candidates than the drift window:
 // bit 0 for the NeighboursFinder's window, bit 1 for the following's.  Both are
 // set when the orders lie too far apart for the 16-bit distances (a cell row of
-// more than 32 k hits): such a row's view is its sorted order with distances of
-// 0 and has no bin starts, so that a row's own hits are read from its view
+// more than 32 k hits).  The view of a row with both is its sorted order, with
+// distances of 0 and no bin starts: a row's own hits are read from its view
 // whatever the flags say, and a flagged row is searched in its cells alone.
 enum : int { kZNFCells = 1, kZFollowCells = 2, kZnz = 8 };
 constexpr int kZShortRow = 65535;  // hits of a row with 16-bit bin starts, at most
