@@ -72,17 +72,10 @@ STAGE_BYTES = {
 # DRAM bytes (read + write) per launch that ncu measured for a kernel on a
 # workload, valid while the kernel's sources hash to the recorded value;
 # otherwise the line says null.
-MEASURED_TRAFFIC = {
-    # the following passes: DRAM counters of the single kernels on the
-    # 1 ms frame (19.70 M clusters at the same 50 kHz density), scaled by the
-    # cluster count (x 241.96 / 19.70) to a launch on the 128-orbit TF
-    ("k_tl_follow<1>", "full_tf"): {"bytes": (2390308000 + 363173888) * 241.96 / 19.70,
-                                    "sources_sha256_16": "3f3b31b4c299e15c",
-                                    "sources": ["k_track.cu", "o2tpc_internal.cuh"]},
-    ("k_tl_follow<-1>", "full_tf"): {"bytes": (2240776000 + 251170560) * 241.96 / 19.70,
-                                     "sources_sha256_16": "3f3b31b4c299e15c",
-                                     "sources": ["k_track.cu", "o2tpc_internal.cuh"]},
-}
+# None now: captures are of the 1 ms frame, and its bytes scaled by the clusters
+# are not the 128-orbit TF's (an earlier build's inward following: 14.2 GB scaled,
+# 25.0 GB measured).
+MEASURED_TRAFFIC = {}
 
 
 def measured_traffic(kernel: str, workload: str):

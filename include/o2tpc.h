@@ -157,7 +157,7 @@ typedef struct {
   /* Captured path (0: off): batches of at most graph_max_tfs TFs (0: 64) and
    * graph_max_clusters clusters run as ONE CUDA graph launch - the whole
    * pipeline captured once and replayed, no host synchronisation inside -
-   * from a device arena allocated at o2tpc_create (about 220 bytes per
+   * from a device arena allocated at o2tpc_create (about 280 bytes per
    * cluster of graph_max_clusters, on top of mem_budget).  A batch whose
    * data exceed the arena's capacities (e.g. far more tracklets than usual)
    * is run again on the regular path; results are the same either way.
@@ -319,8 +319,8 @@ typedef struct {
  * and the centre of gravity of the 3 x 3 cells around it, rounded half up in
  * 1/64 pad and 1/64 time bin.  Runs on `stream` (a cudaStream_t, NULL for the
  * default stream) with scratch from the stream-ordered allocator and returns
- * when the records are written (the buffer may overlap the digits' arrays).  *n_clusters: the number of peaks (also when
- * it exceeds cap).  Returns O2TPC_OK, O2TPC_EINVAL (null pointers, misaligned
+ * when the records are written (the buffer may overlap the digits' arrays).
+ * *n_clusters: the number of peaks (also when it exceeds cap).  Returns O2TPC_OK, O2TPC_EINVAL (null pointers, misaligned
  * records, unsorted or out-of-range digits), O2TPC_ETOOBIG (n >= 2^31, or more
  * peaks than cap: nothing written), O2TPC_ENOMEM, O2TPC_ECUDA. */
 int o2tpc_clusterize(const o2tpc_digits* digits, void* records, uint64_t cap, uint64_t* n_clusters, void* stream);
@@ -342,7 +342,10 @@ typedef struct {
 } o2tpc_ctf_clusters;
 
 /* Decodes a compressed TF (o2tpc_result.ctf) on the host; no device work, no
- * context needed.  Returns O2TPC_OK, O2TPC_EINVAL (not a compressed TF, or
+ * context needed.  From a million symbols on (eight a cluster), up to seven
+ * threads that live for the call share the work, one per half a million symbols
+ * and no more than the host has cores; if none can be started, the caller's does
+ * it alone.  Returns O2TPC_OK, O2TPC_EINVAL (not a compressed TF, or
  * damaged: every chunk's coder must end in its initial state with its bytes
  * used up, and the payloads must end the blob), O2TPC_ENOMEM.  *out is
  * zeroed on error. */
